@@ -18,6 +18,7 @@
 #include "lbkm.h"
 #include "adjoint.cuh"
 #include "kernels.cuh"
+#include "line.cuh"
 #include "model.h"
 
 using namespace lbk;
@@ -45,6 +46,7 @@ struct lbkm {
     int srt;     // the FP32 2-D step takes the single-relaxation-time fast path
     double* partials;
     int grid, tgrid;
+    LinePlan line; // the cut of a 1-D grid
     DevCounters* ctr;
     TneRecord* hist;
     TneRecord* tne_out;
@@ -177,6 +179,26 @@ StepLaunch step_args(const lbkm* h, int from, int stage = 0, const void* src = n
     a.tm_out = &h->tm_store[map_of(a.out)];
     a.srt = h->srt;
     return a;
+}
+
+// `n` forward-Euler steps of a 1-D grid, or one stage of a Runge-Kutta step (as step_args)
+LineArgs line_args(const lbkm* h, int from, int n, int stage = 0, const void* src = nullptr,
+                   double wp = 0.0, double wn = 1.0)
+{
+    const StepLaunch a = step_args(h, from, stage, src, wp, wn);
+    LineArgs l;
+    l.in = a.in;
+    l.out = a.out;
+    l.out_stride = 0;
+    l.nsteps = n;
+    l.prev = a.prev;
+    l.stage = stage;
+    l.wprev = wp;
+    l.wnew = wn;
+    l.partials = a.partials;
+    l.ctr = a.ctr;
+    l.tne_every = a.tne_every;
+    return l;
 }
 
 lbkm_status check_status(lbkm_t h)
@@ -460,11 +482,14 @@ lbkm_status lbkm_create(const lbkm_params* pin, void* cuda_stream, lbkm_t* out)
             if (e != cudaSuccess) return bail(e, "tensor maps");
         }
     }
-    h->grid = step_grid(h->precision, h->recovery, h->two_d, h->nx, h->ny, sbc);
+    h->line = line_plan(h->precision, h->nx);
+    h->grid = h->two_d ? step_grid(h->precision, h->recovery, true, h->nx, h->ny, sbc) : h->line.grid;
     if (h->grid < 1) return bail(cudaGetLastError(), "step grid");
     h->tgrid = tne_grid(h->nx, h->ny);
-    int pg = h->grid > h->tgrid ? h->grid : h->tgrid;
-    if ((e = dmalloc(h, &h->partials, sizeof(double) * TNE_PART * (size_t)pg)) != cudaSuccess)
+    // a 1-D launch leaves the partials of each of its steps
+    const size_t sg = (size_t)h->grid * (h->two_d || p.tne_every == 0 ? 1 : h->line.steps);
+    const size_t pg = sg > (size_t)h->tgrid ? sg : (size_t)h->tgrid;
+    if ((e = dmalloc(h, &h->partials, sizeof(double) * TNE_PART * pg)) != cudaSuccess)
         return bail(e, "partials");
     if ((e = dmalloc(h, &h->ctr, sizeof(DevCounters))) != cudaSuccess) return bail(e, "counters");
     if ((e = cudaMemset(h->ctr, 0, sizeof(DevCounters))) != cudaSuccess) return bail(e, "memset");
@@ -535,9 +560,30 @@ lbkm_status lbkm_init_fields(lbkm_t h, const double* rho, const double* ux, cons
 // With TNE on, a small kernel then turns the step's per-block partials into the record.
 // The three-stage scheme (Shu and Osher's SSP-RK3): u1 = E(u^n) into buf[1-c],
 // u2 = 3/4 u^n + 1/4 E(u1) into buf3, u^{n+1} = 1/3 u^n + 2/3 E(u2) back into buf[c].
-static cudaError_t launch_full_step(const lbkm* h, const void* K, int& c, cudaStream_t st)
+// On a 1-D grid up to line.steps forward-Euler steps go in one launch: `n` comes in as the
+// steps wanted and goes out as the steps launched.
+static cudaError_t launch_full_step(const lbkm* h, const void* K, int& c, int64_t& n, cudaStream_t st)
 {
     const int ts = h->p.time_scheme;
+    if (!h->two_d) {
+        auto go = [&](const LineArgs& a) {
+            return launch_line(h->precision, h->recovery, K, h->line, a, st);
+        };
+        if (ts != 0) n = 1;
+        else if (n > h->line.steps) n = h->line.steps;
+        cudaError_t e = go(line_args(h, c, (int)n, ts == 0 ? 0 : 1));
+        if (e == cudaSuccess && ts == 1) e = go(line_args(h, c, 1, 2, h->buf[1 - c], 0.5, 0.5));
+        if (e == cudaSuccess && ts == 2) {
+            e = go(line_args(h, c, 1, 3, h->buf[1 - c], 0.75, 0.25));
+            if (e == cudaSuccess) e = go(line_args(h, c, 1, 2, h->buf3, 1.0 / 3.0, 2.0 / 3.0));
+        }
+        if (e == cudaSuccess && h->p.tne_every > 0)
+            e = launch_tne_finish_steps(h->partials, h->grid, (int)n, h->hist, h->p.tne_capacity,
+                                        h->p.tne_every, h->ctr, h->p.dx * h->p.dy, st);
+        if (e == cudaSuccess && ts == 0) c = 1 - c;
+        return e;
+    }
+    n = 1;
     const StepLaunch a0 = step_args(h, c, ts == 0 ? 0 : 1);
     cudaError_t e = launch_step(h->precision, h->recovery, h->two_d, K, a0, st);
     if (e == cudaSuccess && ts == 1)
@@ -605,8 +651,10 @@ lbkm_status lbkm_step(lbkm_t h, int64_t n)
             CUDA_TRY(h, cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal));
             int c = h->cur;
             cudaError_t le = cudaSuccess;
-            for (int s = 0; s < GRAPH_CHUNK && le == cudaSuccess; s++)
-                le = launch_full_step(h, K, c, h->capture_stream);
+            for (int64_t left = GRAPH_CHUNK, m; left > 0 && le == cudaSuccess; left -= m) {
+                m = left;
+                le = launch_full_step(h, K, c, m, h->capture_stream);
+            }
             cudaError_t ce = cudaStreamEndCapture(h->capture_stream, &g);
             if (le != cudaSuccess || ce != cudaSuccess) {
                 if (ce == cudaSuccess) cudaGraphDestroy(g);
@@ -622,9 +670,11 @@ lbkm_status lbkm_step(lbkm_t h, int64_t n)
         n -= GRAPH_CHUNK;
         h->host_steps += GRAPH_CHUNK;
     }
-    for (; n > 0; n--) {
-        CUDA_TRY(h, launch_full_step(h, K, h->cur, h->stream));
-        h->host_steps++;
+    while (n > 0) {
+        int64_t m = n;
+        CUDA_TRY(h, launch_full_step(h, K, h->cur, m, h->stream));
+        h->host_steps += m;
+        n -= m;
     }
     return LBKM_OK;
 }
@@ -1079,18 +1129,24 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
     GT(cudaMemsetAsync(pacc, 0, sizeof(double) * (ADJ_NPAR + 2) * G, st));
     GT(cudaMemsetAsync(sctr, 0, sizeof(DevCounters), st));
     GT(cudaMemcpyAsync(K_(0), h->buf[h->cur], SBf, cudaMemcpyDeviceToDevice, st));
-    StepLaunch sl = step_args(h, 0);
+    LineArgs sl = line_args(h, 0, 1);
     sl.ctr = sctr;
     sl.tne_every = 0;
-    StepLaunch sd = sl; // the FP64 step of the recomputed segments
-    sd.grid = step_grid(0, 0, false, nx, 1, h->Kd.sbc);
+    LineArgs sd = sl; // the FP64 steps of the recomputed segments: every state is kept
+    const LinePlan dplan = f32 ? line_plan(0, nx) : h->line;
+    sd.out_stride = (int64_t)(SBd / sizeof(double));
     // forward run in the handle's precision, keeping a state every C steps
-    for (int64_t n = 0; n < N; n++) {
-        sl.in = n == 0 ? (const void*)K_(0) : (const void*)S(n % 2);
-        sl.out = S((n + 1) % 2);
-        GT(launch_step(h->precision, h->recovery, false, model_ptr(h), sl, st));
-        if ((n + 1) % C == 0 && n + 1 < N)
-            GT(cudaMemcpyAsync(K_((n + 1) / C), S((n + 1) % 2), SBf, cudaMemcpyDeviceToDevice, st));
+    const void* fwd = K_(0);
+    int at = 0; // which of S(0), S(1) the run writes next
+    for (int64_t n = 0; n < N;) {
+        const int64_t next = (n / C + 1) * C < N ? (n / C + 1) * C : N;
+        sl.nsteps = (int)(next - n < h->line.steps ? next - n : h->line.steps);
+        n += sl.nsteps;
+        sl.in = fwd;
+        sl.out = n == next && n < N ? K_(n / C) : S(at);
+        GT(launch_line(h->precision, h->recovery, model_ptr(h), h->line, sl, st));
+        fwd = sl.out;
+        at ^= 1;
     }
     AdjArgs a;
     memset(&a, 0, sizeof(a));
@@ -1114,7 +1170,7 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
         a.jacc = jtne;
         return se;
     };
-    if (!f32) GT(seed(S(N % 2)));
+    if (!f32) GT(seed(fwd));
     double *fc = fbA, *fn = fbB, *lc = lbA, *ln = lbB;
     for (int64_t sg = nck - 1; sg >= 0; sg--) {
         const int64_t n0 = sg * C, n1 = (n0 + C < N) ? n0 + C : N;
@@ -1124,10 +1180,11 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
                                 (size_t)NPLANE * h->plane_elems, G, st));
         else
             GT(cudaMemcpyAsync(S(0), K_(sg), SBf, cudaMemcpyDeviceToDevice, st));
-        for (int64_t n = n0; n < (last ? n1 : n1 - 1); n++) {
+        for (int64_t n = n0, end = last ? n1 : n1 - 1; n < end; n += sd.nsteps) {
             sd.in = S(n - n0);
             sd.out = S(n - n0 + 1);
-            GT(launch_step(0, 0, false, &h->Kd, sd, st));
+            sd.nsteps = (int)(end - n < dplan.steps ? end - n : dplan.steps);
+            GT(launch_line(0, 0, &h->Kd, dplan, sd, st));
         }
         if (last) GT(seed(S(n1 - n0)));
         for (int64_t n = n1 - 1; n >= n0; n--) {
@@ -1208,8 +1265,12 @@ lbkm_status lbkm_objective_value(lbkm_t h, const lbkm_objective* ob, double* J,
     };
     // work: fb 16n, lb n (written by the seed kernel), rho_t n, jtne G, jmis G
     const size_t nwork = (size_t)nx * (16 + 1 + 1) + (size_t)2 * G;
-    cudaError_t e = dmalloc(h, &run, SBf * 2);
-    if (e == cudaSuccess && f32) e = dmalloc(h, &seg, SBd * 2);
+    // steps per launch: every FP64 state is wanted, so a launch keeps its steps' states in
+    // one of two sets of `m`; long grids, whose launches are short of nothing, keep one state
+    const LinePlan dplan = f32 ? line_plan(0, nx) : h->line;
+    const int m64 = nx <= 65536 ? dplan.steps : 1;
+    cudaError_t e = dmalloc(h, &run, f32 ? SBf * 2 : SBd * 2 * m64);
+    if (e == cudaSuccess && f32) e = dmalloc(h, &seg, SBd * 2 * m64);
     if (e == cudaSuccess) e = dmalloc(h, &work, sizeof(double) * nwork);
     if (e == cudaSuccess) e = dmalloc(h, &sctr, sizeof(DevCounters));
     if (e != cudaSuccess) {
@@ -1235,59 +1296,65 @@ lbkm_status lbkm_objective_value(lbkm_t h, const lbkm_objective* ob, double* J,
     GT(cudaMemcpyAsync(rho_t, ob->rho_target, sizeof(double) * nx, cudaMemcpyHostToDevice, st));
     GT(cudaMemsetAsync(jtne, 0, sizeof(double) * 2 * G, st));
     GT(cudaMemsetAsync(sctr, 0, sizeof(DevCounters), st));
-    StepLaunch sl = step_args(h, 0);
+    LineArgs sl = line_args(h, 0, 1);
     sl.ctr = sctr;
     sl.tne_every = 0;
-    StepLaunch sd = sl; // the FP64 step of the segments
-    sd.grid = step_grid(0, 0, false, nx, 1, h->Kd.sbc);
+    LineArgs sd = sl; // the FP64 steps whose states the objective reads
+    sd.out_stride = (int64_t)(SBd / sizeof(double));
     AdjArgs a;
     memset(&a, 0, sizeof(a));
     a.fb0 = fb;
     a.lb0 = lb;
     a.jacc = jtne;
     a.jw = ob->w_tne * h->p.dx * h->p.dt;
-    // the TNE term of one FP64 state
-    auto tne_term = [&](const void* state) -> cudaError_t {
-        a.f = static_cast<const double*>(state);
-        return launch_adj_jtne(h->Kd, a, G, st);
-    };
-    // the run in the handle's precision: m steps taken so far, its state in cur
-    const void* cur = h->buf[h->cur];
-    int64_t m = 0;
-    auto advance = [&]() -> cudaError_t {
-        sl.in = cur;
-        sl.out = run + (size_t)(m % 2) * SBf;
-        const cudaError_t se = launch_step(h->precision, h->recovery, false, model_ptr(h), sl, st);
-        cur = sl.out;
-        m++;
-        return se;
+    // `n` FP64 states from `start` on, the TNE term of each, and the state after the last
+    // (`past`: it is wanted); sets: 2 m64 states to keep them in
+    auto segment = [&](const char* start, char* sets, int64_t n, bool past, const void** end) -> cudaError_t {
+        const char* state = start;
+        int set = start == sets ? 1 : 0;
+        for (int64_t k = 0; k < n; k += sd.nsteps) {
+            sd.nsteps = (int)(n - k < m64 ? n - k : m64);
+            sd.in = state;
+            sd.out = sets + (size_t)set * m64 * SBd;
+            const int out = k + sd.nsteps < n || past ? sd.nsteps : sd.nsteps - 1; // states to form
+            const int keep = sd.nsteps;
+            if (out > 0) {
+                sd.nsteps = out;
+                const cudaError_t se = launch_line(0, 0, &h->Kd, dplan, sd, st);
+                sd.nsteps = keep;
+                if (se != cudaSuccess) return se;
+            }
+            for (int j = 0; j < sd.nsteps; j++) {
+                a.f = reinterpret_cast<const double*>(j == 0 ? state : static_cast<char*>(sd.out) + (size_t)(j - 1) * SBd);
+                const cudaError_t se = launch_adj_jtne(h->Kd, a, G, st);
+                if (se != cudaSuccess) return se;
+            }
+            state = static_cast<char*>(sd.out) + (size_t)(sd.nsteps - 1) * SBd;
+            set ^= 1;
+        }
+        *end = state;
+        return cudaSuccess;
     };
     const void* fin = nullptr; // the FP64 state after N steps
     if (!f32) {
-        for (int64_t n = 0; n < N; n++) {
-            GT(tne_term(cur));
-            GT(advance());
-        }
-        fin = cur;
+        GT(segment(static_cast<const char*>(h->buf[h->cur]), run, N, true, &fin));
     } else {
+        const void* cur = h->buf[h->cur]; // the run in the handle's precision
+        int at = 0;
         for (int64_t n0 = 0; n0 < N; n0 += C) {
             const int64_t n1 = (n0 + C < N) ? n0 + C : N;
             const bool last = n1 == N;
             GT(launch_adj_widen(static_cast<const float*>(cur), reinterpret_cast<double*>(seg),
                                 (size_t)NPLANE * h->plane_elems, G, st));
-            for (int64_t n = n0; n < n1; n++) {
-                const int64_t k = n - n0;
-                GT(tne_term(seg + (size_t)(k % 2) * SBd));
-                if (n + 1 < n1 || last) {
-                    sd.in = seg + (size_t)(k % 2) * SBd;
-                    sd.out = seg + (size_t)((k + 1) % 2) * SBd;
-                    GT(launch_step(0, 0, false, &h->Kd, sd, st));
-                }
+            GT(segment(seg, seg, n1 - n0, last, &fin));
+            for (int64_t n = n0; n < n1 && !last; n += sl.nsteps) {
+                sl.in = cur;
+                sl.out = run + (size_t)at * SBf;
+                sl.nsteps = (int)(n1 - n < h->line.steps ? n1 - n : h->line.steps);
+                GT(launch_line(h->precision, h->recovery, model_ptr(h), h->line, sl, st));
+                cur = sl.out;
+                at ^= 1;
             }
-            if (last)
-                fin = seg + (size_t)((n1 - n0) % 2) * SBd;
-            else
-                for (int64_t n = n0; n < n1; n++) GT(advance());
         }
     }
     a.f = static_cast<const double*>(fin);

@@ -1,7 +1,7 @@
 // kernels.cu -- CUDA kernels of the MRT-LBKM step for sm_103a.
 //
-// step_kernel: one fused forward-Euler stage of the FP64 form and of FP32 1-D grids
-// (FP32 2-D grids run march_kernel, march.cu). Each block walks tiles of
+// step_kernel: one fused forward-Euler stage of the FP64 2-D form (FP32 2-D grids run
+// march_kernel, march.cu; 1-D grids line_kernel, line.cu). Each block walks tiles of
 // TX x TY cells (grid-stride loop, grid = SMs x resident blocks). Per tile it
 //   1. stages the 17 planes (f_1..f_16, lambda) of the tile plus a 2-cell halo
 //      in shared memory (coalesced row loads, boundary condition applied by
@@ -21,16 +21,17 @@
 
 #include "cell.cuh"
 #include "kernels.cuh"
+#include "line.cuh"
 #include "reduce.cuh"
 
 namespace lbk {
 
 namespace {
 
-template <typename R, bool TWO_D, int TX, int TY>
+template <typename R, int TX, int TY>
 struct Cfg {
-    static constexpr int H = TWO_D ? 2 : 0;  // halo rows of f (NND radius)
-    static constexpr int H1 = TWO_D ? 1 : 0; // ring rows of macros (grad u)
+    static constexpr int H = 2;  // halo rows of f (NND radius)
+    static constexpr int H1 = 1; // ring rows of macros (grad u)
     static constexpr int SW = TX + 4, SH = TY + 2 * H, PS = SW * SH;
     static constexpr int RW = TX + 2, RH = TY + 2 * H1, RS = RW * RH;
     static constexpr int NT = TX * TY, NW = NT / 32;
@@ -42,11 +43,11 @@ struct Cfg {
     static constexpr size_t smem = off_tmm + (size_t)NW * NMM * sizeof(R);
 };
 
-template <typename R, int REC, bool TWO_D, int TX, int TY>
+template <typename R, int TX, int TY>
 __global__ void __launch_bounds__(TX * TY)
     step_kernel(const ModelConst<R> K, const StepLaunch a)
 {
-    using C = Cfg<R, TWO_D, TX, TY>;
+    using C = Cfg<R, TX, TY>;
     extern __shared__ __align__(16) unsigned char smem[];
     R* sf = reinterpret_cast<R*>(smem);
     R* smac = reinterpret_cast<R*>(smem + C::off_mac); // rho, ux, uy, T  [4][RH][RW]
@@ -86,31 +87,29 @@ __global__ void __launch_bounds__(TX * TY)
             const int p = idx / C::PS;
             const int rem = idx - p * C::PS;
             const int r = rem / C::SW, c = rem - r * C::SW;
-            sf[idx] = ghost_value(K, in, p, x0 - 2 + c, TWO_D ? y0 - C::H + r : y0);
+            sf[idx] = ghost_value(K, in, p, x0 - 2 + c, y0 - C::H + r);
         }
         __syncthreads();
-        if constexpr (TWO_D) {
-            // walls: the staged ghost rows hold copies of the edge fluid row (the
-            // index map clamps); add the non-equilibrium-extrapolation correction
-            if ((K.sbc[2] == 2 || K.sbc[3] == 2) && (y0 - C::H < 0 || y0 + TY + C::H > ny)) {
-                for (int idx = tid; idx < 2 * C::SW; idx += C::NT) {
-                    const int side = idx / C::SW, c = idx - side * C::SW;
-                    if (K.sbc[2 + side] != 2) continue;
-                    const int rs = (side == 0 ? 0 : ny - 1) - (y0 - C::H); // fluid row
-                    if (rs < 0 || rs >= C::SH) continue;
-                    R fl[16], d[16];
+        // walls: the staged ghost rows hold copies of the edge fluid row (the
+        // index map clamps); add the non-equilibrium-extrapolation correction
+        if ((K.sbc[2] == 2 || K.sbc[3] == 2) && (y0 - C::H < 0 || y0 + TY + C::H > ny)) {
+            for (int idx = tid; idx < 2 * C::SW; idx += C::NT) {
+                const int side = idx / C::SW, c = idx - side * C::SW;
+                if (K.sbc[2 + side] != 2) continue;
+                const int rs = (side == 0 ? 0 : ny - 1) - (y0 - C::H); // fluid row
+                if (rs < 0 || rs >= C::SH) continue;
+                R fl[16], d[16];
 #pragma unroll
-                    for (int i = 0; i < 16; i++) fl[i] = sf[i * C::PS + rs * C::SW + c];
-                    wall_correction(K, fl, side, d);
-                    for (int r = 0; r < C::SH; r++) {
-                        const int gy = y0 - C::H + r;
-                        if (side == 0 ? gy >= 0 : gy < ny) continue;
+                for (int i = 0; i < 16; i++) fl[i] = sf[i * C::PS + rs * C::SW + c];
+                wall_correction(K, fl, side, d);
+                for (int r = 0; r < C::SH; r++) {
+                    const int gy = y0 - C::H + r;
+                    if (side == 0 ? gy >= 0 : gy < ny) continue;
 #pragma unroll
-                        for (int i = 0; i < 16; i++) sf[i * C::PS + r * C::SW + c] += d[i];
-                    }
+                    for (int i = 0; i < 16; i++) sf[i * C::PS + r * C::SW + c] += d[i];
                 }
-                __syncthreads();
             }
+            __syncthreads();
         }
         // 2. macros of the tile and its ring
         for (int idx = tid; idx < C::RS; idx += C::NT) {
@@ -120,11 +119,7 @@ __global__ void __launch_bounds__(TX * TY)
 #pragma unroll
             for (int i = 0; i < 16; i++) fl[i] = sf[i * C::PS + s];
             double rho, ux, uy, T;
-            if constexpr (REC == 1)
-                recover_df32(K.cd, K.wd, K.inv_DId, reinterpret_cast<const float*>(fl), rho, ux,
-                             uy, T);
-            else
-                recover_f64(K.cd, K.wd, K.inv_DId, fl, rho, ux, uy, T);
+            recover_f64(K.cd, K.wd, K.inv_DId, fl, rho, ux, uy, T);
             smac[idx] = (R)rho;
             smac[C::RS + idx] = (R)ux;
             smac[2 * C::RS + idx] = (R)uy;
@@ -159,11 +154,8 @@ __global__ void __launch_bounds__(TX * TY)
             const R* suy = smac + 2 * C::RS;
             const R dux_dx = (sux[m0 + 1] - sux[m0 - 1]) * K.half_inv_dx;
             const R duy_dx = (suy[m0 + 1] - suy[m0 - 1]) * K.half_inv_dx;
-            R dux_dy = R(0), duy_dy = R(0);
-            if constexpr (TWO_D) {
-                dux_dy = (sux[m0 + C::RW] - sux[m0 - C::RW]) * K.half_inv_dy;
-                duy_dy = (suy[m0 + C::RW] - suy[m0 - C::RW]) * K.half_inv_dy;
-            }
+            const R dux_dy = (sux[m0 + C::RW] - sux[m0 - C::RW]) * K.half_inv_dy;
+            const R duy_dy = (suy[m0 + C::RW] - suy[m0 - C::RW]) * K.half_inv_dy;
             const R theta = (dux_dx + duy_dy) * K.inv_DI;
             const R shear = duy_dx + dux_dy;
             const R rT = rho * T;
@@ -198,12 +190,8 @@ __global__ void __launch_bounds__(TX * TY)
                 const R cx = K.c[2 * o] * K.inv_dx, cy = K.c[2 * o] * K.inv_dy;
                 adv[i0 + 0] = cx * PX(i0 + 0);
                 adv[i0 + 2] = -cx * NX(i0 + 2);
-                if constexpr (TWO_D) {
-                    adv[i0 + 1] = cy * PY(i0 + 1);
-                    adv[i0 + 3] = -cy * NY(i0 + 3);
-                } else {
-                    adv[i0 + 1] = adv[i0 + 3] = R(0);
-                }
+                adv[i0 + 1] = cy * PY(i0 + 1);
+                adv[i0 + 3] = -cy * NY(i0 + 3);
             }
 #pragma unroll
             for (int o = 0; o < 2; o++) { // diagonal orbits 1, 3
@@ -211,13 +199,8 @@ __global__ void __launch_bounds__(TX * TY)
                 const R cx = K.c[2 * o + 1] * K.inv_dx, cy = K.c[2 * o + 1] * K.inv_dy;
                 R x0p = cx * PX(i0 + 0), x1n = cx * NX(i0 + 1), x2n = cx * NX(i0 + 2),
                   x3p = cx * PX(i0 + 3);
-                R y0p = R(0), y1p = R(0), y2n = R(0), y3n = R(0);
-                if constexpr (TWO_D) {
-                    y0p = cy * PY(i0 + 0);
-                    y1p = cy * PY(i0 + 1);
-                    y2n = cy * NY(i0 + 2);
-                    y3n = cy * NY(i0 + 3);
-                }
+                R y0p = cy * PY(i0 + 0), y1p = cy * PY(i0 + 1), y2n = cy * NY(i0 + 2),
+                  y3n = cy * NY(i0 + 3);
                 adv[i0 + 0] = x0p + y0p;
                 adv[i0 + 1] = y1p - x1n;
                 adv[i0 + 2] = -(x2n + y2n);
@@ -233,10 +216,8 @@ __global__ void __launch_bounds__(TX * TY)
             // lambda: u . grad(lambda) with NND interface values, reaction, clamp
             R la = ux > R(0) ? ux * PX(16) : (ux < R(0) ? ux * NX(16) : R(0));
             la *= K.inv_dx;
-            if constexpr (TWO_D) {
-                R lb = uy > R(0) ? uy * PY(16) : (uy < R(0) ? uy * NY(16) : R(0));
-                la += lb * K.inv_dy;
-            }
+            R lb = uy > R(0) ? uy * PY(16) : (uy < R(0) ? uy * NY(16) : R(0));
+            la += lb * K.inv_dy;
 #undef FV
 #undef PX
 #undef NX
@@ -309,14 +290,14 @@ __global__ void __launch_bounds__(TX * TY)
     }
 }
 
-template <typename R, int REC, bool TWO_D, int TX, int TY>
+template <typename R, int TX, int TY>
 struct StepKernel {
-    using C = Cfg<R, TWO_D, TX, TY>;
+    using C = Cfg<R, TX, TY>;
     // opt in to the dynamic shared memory once per process, before any capture
     static cudaError_t prepare()
     {
         static cudaError_t done = cudaFuncSetAttribute(
-            step_kernel<R, REC, TWO_D, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+            step_kernel<R, TX, TY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
             (int)C::smem);
         return done;
     }
@@ -329,7 +310,7 @@ struct StepKernel {
             cudaGetDevice(&dev);
             cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
             if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                    &per_sm, step_kernel<R, REC, TWO_D, TX, TY>, C::NT, C::smem) != cudaSuccess)
+                    &per_sm, step_kernel<R, TX, TY>, C::NT, C::smem) != cudaSuccess)
                 return -1;
             if (per_sm < 1) per_sm = 1;
         }
@@ -341,17 +322,13 @@ struct StepKernel {
     {
         cudaError_t e = prepare();
         if (e != cudaSuccess) return e;
-        step_kernel<R, REC, TWO_D, TX, TY><<<a.grid, C::NT, C::smem, s>>>(
+        step_kernel<R, TX, TY><<<a.grid, C::NT, C::smem, s>>>(
             *static_cast<const ModelConst<R>*>(K), a);
         return cudaGetLastError();
     }
 };
 
-// tile shapes: 2-D 32 x 8 cells, 1-D 64 cells
-template <typename R, int REC>
-using K2D = StepKernel<R, REC, true, 32, 8>;
-template <typename R, int REC>
-using K1D = StepKernel<R, REC, false, 64, 1>;
+using K2D = StepKernel<double, 32, 8>; // tiles of 32 x 8 cells
 
 // ------------------------------------------------------------ init, macros, TNE
 template <typename R>
@@ -499,19 +476,26 @@ static bool general_sides(const int sbc[4])
 namespace {
 constexpr int FIN_THREADS = 256;
 
-// Block q reduces quantity q of the step's partials (quantity-major: partials[q *
-// nblocks + b]) in a fixed order -- thread t takes blocks t, t + 256, ..., then the
-// lanes in a shuffle tree and the warps in order -- and writes it into the record.
+// Block (q, slot) reduces quantity q of the partials of the launch's slot-th step
+// (quantity-major: partials[(slot * TNE_PART + q) * nblocks + b]) in a fixed order --
+// thread t takes blocks t, t + 256, ..., then the lanes in a shuffle tree and the warps in
+// order -- and writes it into the step's record, if the step was due and its record is not
+// already overwritten by a later one of the same launch.
 __global__ void __launch_bounds__(FIN_THREADS)
     tne_finish_kernel(const double* __restrict__ partials, int nblocks, TneRecord* hist,
-                      int hist_cap, const DevCounters* ctr, double area)
+                      int hist_cap, int tne_every, const DevCounters* ctr, double area)
 {
-    if (!ctr->tne_pending) return;
+    const int slot = blockIdx.y, steps = ctr->tne_pending;
+    if (slot >= steps) return;
+    const int64_t step = ctr->tne_step + slot;
+    if (step % tne_every) return;
+    const int64_t after = (ctr->tne_step + steps - 1) / tne_every - step / tne_every; // later records
+    if (after >= hist_cap) return;
     __shared__ double wsum[FIN_THREADS / 32];
     const int q = blockIdx.x, t = threadIdx.x, lane = t & 31, w = t >> 5;
     const int kind = tne_kind(q);
     double acc = kind == 0 ? 0.0 : (kind == 1 ? DBL_MAX : -DBL_MAX);
-    const double* pq = partials + (size_t)q * nblocks;
+    const double* pq = partials + ((size_t)slot * TNE_PART + q) * nblocks;
     for (int b = t; b < nblocks; b += FIN_THREADS) acc = tne_comb(kind, acc, __ldcg(pq + b));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc = tne_comb(kind, acc, __shfl_xor_sync(0xffffffffu, acc, o));
@@ -519,7 +503,7 @@ __global__ void __launch_bounds__(FIN_THREADS)
     __syncthreads();
     if (t != 0) return;
     for (int k = 1; k < FIN_THREADS / 32; k++) acc = tne_comb(kind, acc, wsum[k]);
-    TneRecord* rec = hist + (ctr->hist_count - 1) % hist_cap;
+    TneRecord* rec = hist + (ctr->hist_count - 1 - after) % hist_cap;
     if (q < TNE_K) rec->sum[q + 4] = acc * area;
     else if (q < 2 * TNE_K) rec->abs_sum[q - TNE_K + 4] = acc * area;
     else if (q < 3 * TNE_K) rec->min[q - 2 * TNE_K + 4] = acc;
@@ -528,36 +512,40 @@ __global__ void __launch_bounds__(FIN_THREADS)
     else rec->d2_sum = acc * area;
     if (q == 0) {
         for (int k = 0; k < 4; k++) rec->sum[k] = rec->abs_sum[k] = rec->min[k] = rec->max[k] = 0.0;
-        rec->step = ctr->tne_step;
+        rec->step = step;
     }
 }
 } // namespace
 
+cudaError_t launch_tne_finish_steps(const double* partials, int grid, int slots, TneRecord* hist,
+                                    int hist_cap, int tne_every, const DevCounters* ctr, double area,
+                                    cudaStream_t s)
+{
+    tne_finish_kernel<<<dim3(TNE_PART, slots), FIN_THREADS, 0, s>>>(partials, grid, hist, hist_cap,
+                                                                    tne_every, ctr, area);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_tne_finish(const StepLaunch& a, cudaStream_t s)
 {
-    tne_finish_kernel<<<TNE_PART, FIN_THREADS, 0, s>>>(a.partials, a.grid, a.hist, a.hist_cap,
-                                                       a.ctr, a.cell_area);
-    return cudaGetLastError();
+    return launch_tne_finish_steps(a.partials, a.grid, 1, a.hist, a.hist_cap, a.tne_every, a.ctr,
+                                   a.cell_area, s);
 }
 
 int step_grid(int precision, int recovery, bool two_d, int nx, int ny, const int sbc[4])
 {
-    if (precision == 0)
-        return two_d ? K2D<double, 0>::grid(nx, ny) : K1D<double, 0>::grid(nx, ny);
-    if (two_d) return march_grid(recovery | (general_sides(sbc) ? 2 : 0), nx, ny);
-    return recovery == 1 ? K1D<float, 1>::grid(nx, ny) : K1D<float, 0>::grid(nx, ny);
+    if (!two_d) return -1; // 1-D grids: line_plan
+    if (precision == 0) return K2D::grid(nx, ny);
+    return march_grid(recovery | (general_sides(sbc) ? 2 : 0), nx, ny);
 }
 
 cudaError_t launch_step(int precision, int recovery, bool two_d, const void* K,
                         const StepLaunch& a, cudaStream_t s)
 {
-    if (precision == 0)
-        return two_d ? K2D<double, 0>::launch(K, a, s) : K1D<double, 0>::launch(K, a, s);
-    if (two_d) {
-        const ModelConst<float>& Kf = *static_cast<const ModelConst<float>*>(K);
-        return launch_march(recovery | (general_sides(Kf.sbc) ? 2 : 0) | (a.srt ? 4 : 0), Kf, a, s);
-    }
-    return recovery == 1 ? K1D<float, 1>::launch(K, a, s) : K1D<float, 0>::launch(K, a, s);
+    if (!two_d) return cudaErrorInvalidValue; // 1-D grids: launch_line
+    if (precision == 0) return K2D::launch(K, a, s);
+    const ModelConst<float>& Kf = *static_cast<const ModelConst<float>*>(K);
+    return launch_march(recovery | (general_sides(Kf.sbc) ? 2 : 0) | (a.srt ? 4 : 0), Kf, a, s);
 }
 
 cudaError_t launch_init(int precision, const ModelConst<double>& Kd, const double* rho,
