@@ -483,7 +483,7 @@ lbkm_status lbkm_create(const lbkm_params* pin, void* cuda_stream, lbkm_t* out)
         }
     }
     h->line = line_plan(h->precision, h->nx);
-    h->grid = h->two_d ? step_grid(h->precision, h->recovery, true, h->nx, h->ny, sbc) : h->line.grid;
+    h->grid = h->two_d ? step_grid(h->precision, h->recovery, h->nx, h->ny, sbc, p.tne_every > 0) : h->line.grid;
     if (h->grid < 1) return bail(cudaGetLastError(), "step grid");
     h->tgrid = tne_grid(h->nx, h->ny);
     // a 1-D launch leaves the partials of each of its steps
@@ -585,15 +585,15 @@ static cudaError_t launch_full_step(const lbkm* h, const void* K, int& c, int64_
     }
     n = 1;
     const StepLaunch a0 = step_args(h, c, ts == 0 ? 0 : 1);
-    cudaError_t e = launch_step(h->precision, h->recovery, h->two_d, K, a0, st);
+    cudaError_t e = launch_step(h->precision, h->recovery, K, a0, st);
     if (e == cudaSuccess && ts == 1)
-        e = launch_step(h->precision, h->recovery, h->two_d, K,
+        e = launch_step(h->precision, h->recovery, K,
                         step_args(h, c, 2, h->buf[1 - c], 0.5, 0.5), st);
     if (e == cudaSuccess && ts == 2) {
-        e = launch_step(h->precision, h->recovery, h->two_d, K,
+        e = launch_step(h->precision, h->recovery, K,
                         step_args(h, c, 3, h->buf[1 - c], 0.75, 0.25), st);
         if (e == cudaSuccess)
-            e = launch_step(h->precision, h->recovery, h->two_d, K,
+            e = launch_step(h->precision, h->recovery, K,
                             step_args(h, c, 2, h->buf3, 1.0 / 3.0, 2.0 / 3.0), st);
     }
     if (e == cudaSuccess && a0.tne_every > 0) e = launch_tne_finish(a0, st);

@@ -532,20 +532,20 @@ cudaError_t launch_tne_finish(const StepLaunch& a, cudaStream_t s)
                                    a.cell_area, s);
 }
 
-int step_grid(int precision, int recovery, bool two_d, int nx, int ny, const int sbc[4])
+int step_grid(int precision, int recovery, int nx, int ny, const int sbc[4], bool tne)
 {
-    if (!two_d) return -1; // 1-D grids: line_plan
     if (precision == 0) return K2D::grid(nx, ny);
-    return march_grid(recovery | (general_sides(sbc) ? 2 : 0), nx, ny);
+    return march_grid(recovery | (general_sides(sbc) ? 2 : 0) | (tne ? 8 : 0), nx, ny);
 }
 
-cudaError_t launch_step(int precision, int recovery, bool two_d, const void* K,
-                        const StepLaunch& a, cudaStream_t s)
+cudaError_t launch_step(int precision, int recovery, const void* K, const StepLaunch& a,
+                        cudaStream_t s)
 {
-    if (!two_d) return cudaErrorInvalidValue; // 1-D grids: launch_line
     if (precision == 0) return K2D::launch(K, a, s);
     const ModelConst<float>& Kf = *static_cast<const ModelConst<float>*>(K);
-    return launch_march(recovery | (general_sides(Kf.sbc) ? 2 : 0) | (a.srt ? 4 : 0), Kf, a, s);
+    return launch_march(recovery | (general_sides(Kf.sbc) ? 2 : 0) | (a.srt ? 4 : 0) |
+                            (a.tne_every > 0 ? 8 : 0),
+                        Kf, a, s);
 }
 
 cudaError_t launch_init(int precision, const ModelConst<double>& Kd, const double* rho,

@@ -58,13 +58,14 @@ struct StepLaunch {
 cudaError_t launch_tne_finish(const StepLaunch& a, cudaStream_t s);
 
 // precision: 0 = FP64, 1 = FP32; recovery: 0 = FP64, 1 = double-float (FP32 only)
-cudaError_t launch_step(int precision, int recovery, bool two_d, const void* K,
-                        const StepLaunch& a, cudaStream_t s);
+// (2-D grids; 1-D grids: launch_line, line.cuh)
+cudaError_t launch_step(int precision, int recovery, const void* K, const StepLaunch& a,
+                        cudaStream_t s);
 // Blocks to launch for a step on this grid (multiple of the SM count times the
 // resident blocks per SM, capped by the number of tiles).
 // sbc: the side conditions (walls, Dirichlet or specular sides select the general
-// variant of the FP32 marching kernel)
-int step_grid(int precision, int recovery, bool two_d, int nx, int ny, const int sbc[4]);
+// variant of the FP32 marching kernel); tne: the handle keeps TNE records
+int step_grid(int precision, int recovery, int nx, int ny, const int sbc[4], bool tne);
 
 cudaError_t launch_init(int precision, const ModelConst<double>& Kd, const double* rho,
                         const double* ux, const double* uy, const double* T, const double* lam,
@@ -141,7 +142,7 @@ cudaError_t launch_adj_rho0(const ModelConst<double>& K, const AdjArgs& a, doubl
 cudaError_t launch_adj_widen(const float* in, double* out, size_t n, int grid, cudaStream_t s);
 
 // FP32 2-D step: y-marching strips, two cells per thread (march.cu)
-// mode = recovery | (general side conditions << 1)
+// mode = recovery | (general side conditions << 1) | (single relaxation time << 2) | (TNE << 3)
 // Tensor maps of an FP32 state buffer for the step kernel's bulk tensor copies: loads of
 // a box of BW + 8 columns x 2 rows x 17 planes, stores of BW x 2 x 17.
 cudaError_t march_tensor_maps(const void* state, int nx, int ny, int pitch, int64_t plane,

@@ -183,6 +183,22 @@ __device__ __forceinline__ void row_source(const ModelConst<float>& K, int r, in
     }
 }
 
+// A strip that the grid does not fill: threads past pair `last_pair` (the first pair beyond
+// the grid, whose columns the side map fills) stand on that pair's cells, so no staged column
+// from last_column on is read. (Filling the whole box instead took up to 126 four-byte copies
+// per thread and row pair: 20 us an iteration on the last strip of a 1030-column grid,
+// against 4.4 us on a full strip.)
+__device__ __forceinline__ int last_pair(int nx, int x0)
+{
+    const int p = (nx - 1 - x0) / 2 + 1;
+    return p < BW / 2 - 1 ? p : BW / 2 - 1;
+}
+__device__ __forceinline__ int last_column(int nx, int x0)
+{
+    const int c = x0 + 2 * last_pair(nx, x0) + 4;
+    return c < x0 + BW + 2 ? c : x0 + BW + 2;
+}
+
 // Issue the copies of staged rows ra, ra+1 (pair mbarrier mb) for the strip at x0;
 // rows above rmax are not needed. A pair whose rows and staged columns all lie inside
 // the grid arrives by one tensor copy (thread 0). Otherwise warp 0: one bulk copy per
@@ -250,10 +266,8 @@ __device__ __forceinline__ void issue_pair(const float* __restrict__ in, float* 
         }
         const int ft = tid - 64; // 0..63
         // tasks: (row, plane, side) with side 0 = columns [x0-2, cs), side 1 = columns
-        // [max(ce, x0-2), min(nx+4, x0+BW+2)) (the ghost columns active cells read, and
-        // two more that only an inactive neighbour reads; with periodic or zero-gradient
-        // sides every column up to x0+BW+2, so that a cell past the grid holds a real
-        // cell's values); Dirichlet rows: every column
+        // [max(ce, x0-2), last_column) (the ghost columns active cells read, and the pair of
+        // cells past the grid with its stencil); Dirichlet rows: every column
         for (int task = ft; task < 4 * NPLANE; task += 64) {
             const int side = task & 1, rp = task >> 1;
             const int r = ra + rp / NPLANE, p = rp % NPLANE;
@@ -267,7 +281,7 @@ __device__ __forceinline__ void issue_pair(const float* __restrict__ in, float* 
                 c1 = side ? x0 + BW + 2 : x0 + BW / 2;
             } else {
                 c0 = side ? (ce > x0 - 2 ? ce : x0 - 2) : x0 - 2;
-                c1 = side ? (!GEN ? x0 + BW + 2 : (K.nx + 4 < x0 + BW + 2 ? K.nx + 4 : x0 + BW + 2)) : cs;
+                c1 = side ? last_column(K.nx, x0) : cs;
                 if (!side && ce <= cs) c1 = x0 - 2; // no bulk copy: side 1 takes the row
                 if (side && ce <= cs) c0 = x0 - 2;
             }
@@ -332,11 +346,10 @@ struct Mac {
 // or double-float); u, v also into the (u, v) ring, with the halo columns x0-1 and
 // x0+BW (plain FP32 velocity, used only in grad u) by the first and last thread.
 template <int REC>
-__device__ __forceinline__ Mac recover_row(float* smem_f, float* ring, int r, int t,
+__device__ __forceinline__ Mac recover_row(float* smem_f, float* ring, int r, int lx,
                                            const ModelConst<float>& K, const DfConst& C, int& bad,
                                            bool act0, bool act1)
 {
-    const int lx = XO + 2 * t;
     V2 f[16];
 #pragma unroll
     for (int i = 0; i < 16; i++) f[i] = ldv(plane_row(ring, i, r) + lx);
@@ -348,6 +361,7 @@ __device__ __forceinline__ Mac recover_row(float* smem_f, float* ring, int r, in
     float* vr = uv_row(smem_f, r, 1);
     *reinterpret_cast<float2*>(ur + lx) = o.ux.v;
     *reinterpret_cast<float2*>(vr + lx) = o.uy.v;
+    const int t = threadIdx.x & 63;
     if (t == 0 || t == 63) {
         const int hx = t == 0 ? XO - 1 : XO + BW;
         float g[16], hu, hv;
@@ -380,20 +394,19 @@ __device__ __forceinline__ void acc_exact(V2& s, float& c, V2 x)
 }
 
 // ---------------- the update of one row by one warp pair -------------------------
-// Row y, the thread's cells x0 + 2t and x0 + 2t + 1 (active when act0 / act1), macros
-// mc recovered in the previous iteration; the results go to the output rows ob
-// (17 planes of BW floats). TNE: the row's TNE statistics join the thread's sums. With
-// periodic or zero-gradient sides (!GEN) a cell past the grid's last column holds a real
-// cell's values (staging fills the whole box through the side map), so the statistics
-// run without a branch: the sums take Delta_k times the lane mask am (1 active, 0 not),
-// the extremes the unmasked values. With general sides they take the active cells only.
+// Row y, the thread's two cells (element lx of a staged row; active when act0 / act1), macros
+// mc recovered in the previous iteration; the results go to ob, the thread's
+// place in the output rows (17 planes of 2 x BW floats). TNE: the row's TNE statistics join the thread's sums. With
+// periodic or zero-gradient sides (!GEN) a thread past the grid's last column stands on a
+// real cell's values (last_pair), so the statistics run without a branch: the sums take
+// Delta_k times the lane mask am (1 active, 0 not), the extremes the unmasked values. With
+// general sides they take the active cells only.
 template <int REC, bool AVG, bool SRT, bool TNE, bool GEN>
 __device__ __forceinline__ void update_row(float* smem_f, float* ring, float* ob, int y, int x0,
-                                           int t, const ModelConst<float>& K, const StepLaunch& a,
-                                           const Mac& mc, bool act0, bool act1, V2 am, TneAcc& acc,
-                                           float* tmin, float* tmax)
+                                           int lx, const ModelConst<float>& K,
+                                           const StepLaunch& a, const Mac& mc, bool act0, bool act1,
+                                           V2 am, TneAcc& acc, float* tmin, float* tmax)
 {
-    const int lx = XO + 2 * t;
     const float dt = K.dt;
     const V2 rho = mc.rho, ux = mc.ux, uy = mc.uy, T = mc.T;
     float* r0 = srow(ring, y);
@@ -507,7 +520,7 @@ __device__ __forceinline__ void update_row(float* smem_f, float* ring, float* ob
 
     // results into the output rows; a later SSP Runge-Kutta stage (AVG) writes
     // wp * u^n + wn * E(in), u^n read from prev at the cell's own position
-    const int64_t g = (int64_t)y * K.pitch + x0 + 2 * t;
+    const int64_t g = (int64_t)y * K.pitch + x0 + 2 * (int)(threadIdx.x & 63);
     const float* pv = static_cast<const float*>(a.prev);
     const float wp = (float)a.wprev, wn = (float)a.wnew;
     auto store = [&](int i, V2 v) {
@@ -517,7 +530,7 @@ __device__ __forceinline__ void update_row(float* smem_f, float* ring, float* ob
             else if (act0)
                 v = V2(fmaf(wp, pv[i * K.plane + g], wn * v.x()), 0.f);
         }
-        *reinterpret_cast<float2*>(ob + i * 2 * BW + 2 * t) = v.v;
+        *reinterpret_cast<float2*>(ob + i * 2 * BW) = v.v;
     };
 
     // lambda: u . grad(lambda) with NND interface values
@@ -614,10 +627,10 @@ __global__ void __launch_bounds__(MT, 2)
     const uint32_t mbar0 = smem_addr(smem + OFF_MBAR);
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int wpair = warp >> 1, t = tid & 63, lx = XO + 2 * t;
+    const int wpair = warp >> 1;
     const int nx = K.nx, ny = K.ny;
     const float* __restrict__ in = static_cast<const float*>(a.in);
-    float* ob = obuf + wpair * BW;
+    float* ob = obuf + wpair * BW + 2 * (tid & 63); // the thread's cells in the output rows
 
     const DfConst C = df_constants(K);
     const int64_t step = a.ctr->step;
@@ -648,7 +661,8 @@ __global__ void __launch_bounds__(MT, 2)
     for (int s = blockIdx.x; s < nstrips; s += gridDim.x) {
         const int x0 = (s / nsy) * BW, y0 = (s % nsy) * strip_rows;
         const int yend = y0 + strip_rows < ny ? y0 + strip_rows : ny;
-        const int cx = x0 + 2 * t;
+        const int t = tid & 63, cx = x0 + 2 * t, tl = last_pair(nx, x0);
+        const int lx = XO + 2 * (t < tl ? t : tl); // the thread's cells in a staged row
         const bool act0 = cx < nx, act1 = cx + 1 < nx;
         const V2 am(act0 ? 1.f : 0.f, act1 ? 1.f : 0.f); // lanes whose cells are in the grid
         const int npairs = (yend - y0 + 5) / 2; // rows y0-2 .. yend+1
@@ -668,14 +682,14 @@ __global__ void __launch_bounds__(MT, 2)
         wait_pair(q0);
         wait_pair(q0 + 1);
         // walls: ghost rows among rows y0-2 .. y0+1 (warp pair 0: y0-1, y0+1; 1: y0-2, y0)
-        if constexpr (GEN) {
+        if (GEN && x0 + lx - XO == cx) { // one thread per pair of cells
             wall_fix<GEN>(ring, wpair ? y0 - 2 : y0 - 1, K, lx);
             wall_fix<GEN>(ring, wpair ? y0 : y0 + 1, K, lx);
         }
         __syncthreads();
         // rho, u, T of rows y0 (pair 0) and y0+1 (pair 1), u, v of row y0-1 (pair 0)
-        Mac cur = recover_row<REC>(smem_f, ring, y0 + wpair, t, K, C, bad, act0, act1);
-        if (wpair == 0) (void)recover_row<REC>(smem_f, ring, y0 - 1, t, K, C, bad, act0, act1);
+        Mac cur = recover_row<REC>(smem_f, ring, y0 + wpair, lx, K, C, bad, act0, act1);
+        if (wpair == 0) (void)recover_row<REC>(smem_f, ring, y0 - 1, lx, K, C, bad, act0, act1);
         if (__syncthreads_or(timeout)) break;
 
         bool stop = false;
@@ -685,17 +699,17 @@ __global__ void __launch_bounds__(MT, 2)
             if (y + 2 <= yend + 1) wait_pair(q0 + k + 2);
             const int rr = y + 2 + wpair; // the row this pair recovers
             if constexpr (GEN)
-                if (rr <= yend + 1) wall_fix<GEN>(ring, rr, K, lx);
+                if (rr <= yend + 1 && XO + 2 * (int)(threadIdx.x & 63) == lx) wall_fix<GEN>(ring, rr, K, lx);
             Mac nxt = cur;
-            if (rr <= yend) nxt = recover_row<REC>(smem_f, ring, rr, t, K, C, bad, act0, act1);
+            if (rr <= yend) nxt = recover_row<REC>(smem_f, ring, rr, lx, K, C, bad, act0, act1);
             if (warp == 1) bulk_wait_read_all(); // the output buffer is free again
             if (__syncthreads_or(timeout)) {
                 stop = true;
                 break;
             }
             if (y + wpair < yend)
-                update_row<REC, AVG, SRT, TNE, GEN>(smem_f, ring, ob, y + wpair, x0, t, K, a, cur,
-                                                    act0, act1, am, acc, tmin, tmax);
+                update_row<REC, AVG, SRT, TNE, GEN>(smem_f, ring, ob, y + wpair, x0, lx, K, a, cur, act0,
+                                                    act1, am, acc, tmin, tmax);
             cur = nxt;
             fence_async_shared(); // the output rows are read by the bulk stores
             __syncthreads();
@@ -858,27 +872,42 @@ void launch_variant(bool avg, bool srt, const ModelConst<float>& K, const StepLa
 
 } // namespace
 
-// Blocks resident on the whole GPU, and the strip height: the number of strips per
-// column of the grid is chosen so that the strips fill whole waves of the resident
-// blocks while each strip stays long compared with its prologue (four rows staged and
-// three recovered before the first update).
-// mode = recovery | (general boundaries << 1) | (single relaxation time << 2): the
-// general variant carries walls, Dirichlet and specular sides, the plain one only index
+// Blocks resident on the whole GPU, and the strip height.
+// mode = recovery | (general boundaries << 1) | (single relaxation time << 2) | (TNE << 3):
+// the general variant carries walls, Dirichlet and specular sides, the plain one only index
 // maps; the single-relaxation-time variant exists for the plain forward-Euler step.
+//
+// The blocks take strips in turn, so a launch lasts as long as the rounds of strips over the
+// resident blocks times what one strip takes: half its rows in iterations and a prologue
+// (four rows staged, three recovered) worth MARCH_PROLOGUE of one; a block alone on its SM
+// runs faster than one of two, and few long strips end less evenly than many short ones
+// (MARCH_TAIL of an iteration per iteration of a strip). The height with the least sum is
+// taken; with TNE a strip keeps to 64 rows, over which its plain FP32 sums of d and d^2 run.
+// Measured, us per step (rows: 64, or fewer to give every block a strip, as the rule before
+// had it; then this rule's): 4096^2 with TNE 64 1193, 54 1148; without 64 1011, 72 970 (108
+// 976, 216 1011); 2048^2 equal rates 64 306, 54 260 (108 274); 1030 x 517 8 43.8, 16 43.2 (12
+// 51.7, 32 67.1); 3000 x 130 8 67.3, 12 53.9; 130 x 2900 8 84.6, 20 59.8; 300 x 100 per-side
+// 8 27.5, 2 21.7; 96 x 96 8 26.4, 2 12.9.
+constexpr double MARCH_PROLOGUE = 1.3, MARCH_ALONE = 0.65, MARCH_TAIL = 0.15;
+
 void march_plan(int mode, int nx, int ny, int* grid, int* strip_rows)
 {
     const int G = resident_blocks(mode);
     const int nsx = (nx + BW - 1) / BW;
-    // 64-row strips (4096^2, Gcell/s: 16 rows 14.15, 32 rows 14.97, 48 rows 15.28,
-    // 64 rows 15.30, 96 rows 14.61); smaller grids use shorter strips so that every
-    // resident block gets work
-    int rows = 64;
-    while (rows > 8 && (long)nsx * ((ny + rows - 1) / rows) < G) rows /= 2;
-    if (rows > ny) rows = ny;
+    const int even = (ny + 1) & ~1, cap = (mode & 8) && even > 64 ? 64 : even;
+    int rows = 2;
+    double best = 1e300;
+    for (int r = 2; r <= cap && G > 0; r += 2) {
+        const long strips = (long)nsx * ((ny + r - 1) / r), rounds = (strips + G - 1) / G;
+        const double t = rounds * (r / 2 + MARCH_PROLOGUE) * (2 * strips <= G ? MARCH_ALONE : 1.0) +
+                         MARCH_TAIL * (r / 2);
+        if (t <= best) best = t, rows = r;
+    }
     if (const char* env = getenv("LBKM_MARCH_ROWS")) { // tuning override (even)
         const int r = (atoi(env) + 1) & ~1;
-        if (r >= 2) rows = r < ny ? r : ny;
+        if (r >= 2) rows = r;
     }
+    if (rows > ny) rows = ny;
     const long strips = (long)nsx * ((ny + rows - 1) / rows);
     *grid = G < 0 ? -1 : (int)(strips < G ? strips : G);
     *strip_rows = rows;
