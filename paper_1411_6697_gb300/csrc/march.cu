@@ -259,7 +259,8 @@ __device__ __forceinline__ void issue_pair(const float* __restrict__ in, float* 
         // of the pair is a Dirichlet ghost row
         bool need = x0 - 2 < cs || ce < x0 + BW + 2;
         if constexpr (GEN)
-            need = need || (ra < 0 && K.sbc[2] == 3) || (ra + 1 >= K.ny && ra + 1 <= rmax && K.sbc[3] == 3);
+            need = need || (ra < 0 && K.sbc[2] == 3) ||
+                   (K.sbc[3] == 3 && ra <= rmax && (ra >= K.ny || (ra + 1 == K.ny && ra + 1 <= rmax)));
         if (!need) {
             cp_arrive_noinc(mb);
             return;
