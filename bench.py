@@ -36,12 +36,12 @@ import lbkm_inputs as li  # noqa: E402
 
 N_CELLS_SIDE = 4096
 BYTES_PER_CELL = {"f32": 136, "f64": 272}  # read + write of 16 f + lambda
-# FP64 operations per cell update of the plain FP64 step kernel (step_kernel<double>, 2-D),
+# FP64 operations per cell update of the plain FP64 step kernel (tile_kernel<double>, 2-D),
 # from ncu's executed-instruction counters on a 1024 x 1024 grid: 2 per DFMA, 1 per DADD and
 # DMUL (profiles/step_kernel_fp64_reactive2d.md)
-F64_FLOP_PER_CELL = 911.5
+F64_FLOP_PER_CELL = 779.3
 F64_FLOP_SOURCE = ("ncu sm__sass_thread_inst_executed_op_{dfma,dadd,dmul}_pred_on on one step of "
-                   "a 1024 x 1024 reactive field with TNE: 213.96 DFMA + 375.76 DADD + 107.87 DMUL "
+                   "a 1024 x 1024 reactive field with TNE: 198.06 DFMA + 300.10 DADD + 83.04 DMUL "
                    "per cell")
 
 METRIC = "Mcell-updates/s (16 f_i)"
@@ -74,11 +74,11 @@ def measured_peak():
         return 6800.0, "fallback"
 
 
-# the FP32 2-D step runs march_kernel (march.cu); FP64 and 1-D grids run step_kernel
+# the FP32 2-D step runs march_kernel (march.cu); the FP64 2-D step tile_kernel (tile.cu)
 STEP_KERNEL_SOURCES = {
     "march": ("march.cu", "pair.cuh", "vec2.cuh", "reduce.cuh", "cell.cuh", "kernels.cuh",
               "model.h"),
-    "step": ("kernels.cu", "cell.cuh", "kernels.cuh", "model.h", "reduce.cuh"),
+    "step": ("tile.cu", "cellops.cuh", "cell.cuh", "pair.cuh", "kernels.cuh", "model.h", "reduce.cuh"),
     "batch": ("batch.cu", "cell.cuh", "pair.cuh", "vec2.cuh", "kernels.cuh", "model.h"),
 }
 PROFILE = {"march": "march_kernel_reactive2d.md", "step": "step_kernel_fp64_reactive2d.md",
@@ -755,7 +755,7 @@ def main():
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": traffic,
                      "peak_kind": peak_kind, "kernel": ("march_kernel<%d> (f32)" % rec) if kernel == "march"
-                     else "step_kernel (%s)" % tag,
+                     else "tile_kernel (%s)" % tag,
                      "algorithmic_bytes_per_launch": alg_bytes,
                      "duration": "CUDA events over the timed steps, each the step kernel "
                                  "and the few-microsecond TNE finish kernel"},
