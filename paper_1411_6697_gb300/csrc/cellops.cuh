@@ -258,6 +258,56 @@ __device__ __forceinline__ int source(int j, int n, const int32_t* sbc, int side
     return map_index(j, n, code == 0 ? 0 : 1);
 }
 
+// Stages rows y0 .. y0 + SH - 1 and columns x0 .. x0 + 31 + EXTRA of all NPL planes, row r by
+// warp r % TW: lane c copies the columns c and 32 + c. Sources that lie in the grid (all but
+// Dirichlet ghosts) arrive asynchronously; `mirror(p)` is the plane whose v_y is reversed. A
+// row without Dirichlet ghosts takes the branch-free loop.
+template <int NPL, int SH, int SW, int TW, bool TWO_D, typename R, typename Mirror>
+__device__ __forceinline__ void stage_tile(const R* __restrict__ in, R* sf, int x0, int y0, int nx, int ny,
+                                           int pitch, int64_t plane, const int32_t* sides, const R (*sfeq)[NPL],
+                                           Mirror mirror)
+{
+    constexpr int PS = SH * SW, EXTRA = SW - 32;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    bool m_;
+    const int c0 = source(x0 + lane, nx, sides, 0, m_);
+    const int c1 = lane < EXTRA ? source(x0 + 32 + lane, nx, sides, 0, m_) : 0;
+    const bool inside = __all_sync(0xffffffffu, c0 >= 0 && c1 >= 0);
+    for (int r = warp; r < SH; r += TW) {
+        bool mir = false;
+        const int gy = TWO_D ? source(y0 + r, ny, sides, 2, mir) : 0;
+        R* dst = sf + r * SW + lane;
+        const R* src = in + (int64_t)(gy < 0 ? 0 : gy) * pitch;
+        if (inside && gy >= 0 && !mir) {
+            const R *s0 = src + c0, *s1 = src + c1;
+#pragma unroll
+            for (int p = 0; p < NPL; p++) {
+                cp1(dst + p * PS, s0);
+                s0 += plane;
+            }
+            if (lane < EXTRA) {
+#pragma unroll
+                for (int p = 0; p < NPL; p++) {
+                    cp1(dst + p * PS + 32, s1);
+                    s1 += plane;
+                }
+            }
+            continue;
+        }
+        const int g0 = gy < 0 ? gy : c0, g1 = gy < 0 ? gy : c1; // a Dirichlet row: all of it
+#pragma unroll 1
+        for (int p = 0; p < NPL; p++) {
+            const R* sp = src + (mir ? mirror(p) : p) * plane;
+            if (g0 >= 0) cp1(dst + p * PS, sp + g0);
+            else dst[p * PS] = sfeq[-1 - g0][p];
+            if (lane < EXTRA) {
+                if (g1 >= 0) cp1(dst + p * PS + 32, sp + g1);
+                else dst[p * PS + 32] = sfeq[-1 - g1][p];
+            }
+        }
+    }
+}
+
 // ---- per-warp TNE statistics ----------------------------------------------------
 // Row k of td (stride ld) holds Delta_{k+5} (k < 12), d and d^2 of the block's cells. The
 // warp's lanes take the 26 sums over the warp's own cells (those in `mask`), one quantity

@@ -1,15 +1,21 @@
 // d2v24.cu -- the paper's own 24-velocity model (D2V24, Sec. II Eqs. (25)-(27)):
 // kernels and the C ABI of include/lbkm24.h.
 //
-// The step is one fused kernel per time step, one thread per cell: the 24 f_i of
-// the cell and of its NND stencil (radius 2 in x and y) are read through the
-// read-only data cache; rho, u, T of the block's cells and a one-cell rim are formed
-// once, in FP64 (an FP32 state sums its conserved moments as exact double-floats on
-// the FP32 pipes first), and kept in shared memory; the equilibrium moments, the 20
-// non-conserved moments, the relaxation, the back-transform, the chemical term of
-// Eq. (24) and the NND update run in the storage type R (FP64 or FP32); the TNE
-// partials of the state being read are reduced per block when due (sums in FP64,
-// extremes exactly in R), and an 82-block kernel turns them into one history record.
+// The step is one fused kernel per time step, one thread per cell, in tiles (step_kernel):
+// the 25 planes of a tile and its two-cell halo are staged in shared memory by asynchronous
+// copies; rho, u, T of the tile's cells and u of its rim are formed in FP64 (an FP32 state sums
+// its conserved moments as exact double-floats on the FP32 pipes first); the 20 non-conserved
+// moments less their equilibrium, the relaxation, the back-transform, the chemical term of
+// Eq. (24) and the NND update run in the storage type R (FP64 or FP32); the TNE statistics of
+// the state being read gather per warp (sums in FP64 or as exact FP32 pairs, extremes exactly),
+// and an 82-block kernel turns them into one history record.
+//
+// What bounds it. FP32: instruction issue (60 % of the slots; about 3500 instructions per warp
+// and step, half of them the exact sums of the recovery). FP64: the FP64 unit (cellops.cuh);
+// 720 of its instructions per warp and 1-D step, 240 more where a cell of the warp reacts.
+// Measured per step, against one thread per cell reading its stencil through the cache, every
+// sum normalised, the reaction in FP64 divisions and exponentials throughout: 2048^2 FP32 1.95
+// -> 0.60 ms, the 5000-cell detonation FP64 54 -> 37 us, FP32 12.6 -> 6.6 us.
 //
 // M and M^-1 act in block form: butterflies inside each orbit of four velocities
 // (axis: f1+f3, f2+f4, f1-f3, f2-f4; diagonal: the sum and the three sign patterns)
@@ -30,26 +36,27 @@
 #include <string>
 #include <vector>
 
-#include "cell.cuh"
+#include "cellops.cuh"
 #include "kernels.cuh"
 #include "lbkm24.h"
-#include "pair.cuh"
 
 namespace v24 {
 
 using lbk::DevCounters;
+using lbk::ad;
+using lbk::dbits;
 using lbk::f2d_exact;
+using lbk::fm;
 using lbk::map_index;
-using lbk::nnd_neg;
-using lbk::nnd_pos;
+using lbk::mu;
 using lbk::reaction_increment;
+using lbk::sub;
 
 constexpr int NV = 24;
 constexpr int NP = NV + 1;       // planes: f_1..f_24, lambda
 constexpr int TK = NV - 4;       // non-conserved moments Delta_5..Delta_24
 constexpr int NQ = 4 * TK + 2;   // TNE quantities: sum, |sum|, min, max of each, d, d^2
-constexpr int BT = 128;          // threads per block: 128 x 1 or 32 x 1 (1-D grids), 32 x 4
-constexpr int MAC_CELLS = 390;   // macros staged per block: (128 + 2) x 3 >= (32 + 2) x 6
+constexpr int BT = 128;          // threads per block of tne_kernel: 128 x 1 or 32 x 1 (1-D), 32 x 4
 constexpr int GRAPH_CHUNK = 32;  // even: a replay leaves the ping-pong index unchanged
 
 // signs of v_x, v_y of velocity i = 8 g + 4 o + j (speed group g, o = 0 axis orbit with
@@ -92,9 +99,14 @@ template <typename R>
 struct Model {
     R Bf[NB];  // forward blocks, row-major [moment][component] per sector
     R Bi[NB];  // their inverses, row-major [component][moment]
+    R Bis[NB]; // the inverses with the butterfly scales (1/2 axis, 1/4 diagonal orbits) folded in
     R vx[NV], vy[NV], eta2[NV], S[NV];
     R vxs[NV], vys[NV];              // v_x / dx and v_y / dy in R
-    R dt_r, inv_dx_r, inv_dy_r, hdx_r, hdy_r, I_r, DI_r, A8c_r, A9c_r; // constants in R
+    R dt_r, inv_dx_r, inv_dy_r, hdx_r, hdy_r, I_r, DI_r, inv_DI_r, A8c_r, A9c_r; // constants in R
+    R c_r[6], chem_o[6];             // of each orbit: its speed, I v^2 + eta^2
+    double kchem;                    // Q / (dt I (D + I))
+    int32_t sides[4];                // condition of each side: 0 periodic, 1 zero gradient, 2
+                                     // wall, 3 Dirichlet, 4 specular
     double vxd[NV], vyd[NV], wd[NV]; // FP64 copies for the conserved sums
     double cd[6], wod[6];            // speed and v^2 + eta^2 of each orbit (FP64)
     float cdh[6], cdl[6], wdh[6], wdl[6]; // the same split into hi + lo FP32 pairs
@@ -103,11 +115,7 @@ struct Model {
     double dt, inv_dx, inv_dy;
     int nx, ny, pitch, bc_x, bc_y, pad_;
     int64_t plane;
-    // per-side conditions (bc_x or bc_y = LBKM_BC_SIDES) of the sides x = 0, x = nx,
-    // y = 0, y = ny: 1 zero gradient, 3 Dirichlet (ghost cells hold sfeq: the
-    // equilibrium f of the side's state and its lambda), 4 specular (y sides: the mirror
-    // cell across the face with v_y reversed); 0 for a periodic direction
-    int sbc[4];
+    // Dirichlet sides: ghost cells hold the equilibrium f of the side's state and its lambda
     R sfeq[4][NP];
     // walls (code 2, y sides) by non-equilibrium extrapolation: the ghost rows take the
     // edge row's f plus wall[side][i][x] = [M^-1 (f_hat^eq(rho, u_w, T_w) -
@@ -145,6 +153,14 @@ __device__ __forceinline__ double to_r<double>(double x) { return x; }
 template <>
 __device__ __forceinline__ float to_r<float>(double x) { return lbk::d2f_rn(x); }
 
+// the same for values known to be finite, branch-free
+template <typename R>
+__device__ __forceinline__ R to_fast(double x);
+template <>
+__device__ __forceinline__ double to_fast<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float to_fast<float>(double x) { return lbk::d2f_fast(x); }
+
 __device__ __forceinline__ double to_f64(double x) { return x; }
 // exact, on the integer pipe (the FP64 unit runs at 1/58 of the FP32 rate on GB300)
 __device__ __forceinline__ double to_f64(float x) { return f2d_exact(x); }
@@ -159,56 +175,19 @@ __host__ __device__ __forceinline__ int mirror24(int i)
     return 4 * o + jm;
 }
 
-// Value of plane i (0..23 f, 24 lambda) at cell (x, y), which may lie up to two cells
-// outside the grid: periodic or zero-gradient directions map the index; with per-side
-// conditions a Dirichlet side (a y side first, as corners are never read by the
-// cross-shaped stencil) gives its equilibrium value, a specular y side the mirror
-// cell's value of the velocity with v_y reversed, an outflow side the edge cell's.
-template <typename R>
-__device__ __forceinline__ R fval(const Model<R>& K, const R* __restrict__ in, int i, int x, int y)
-{
-    const int cx = (x >= 0 && x < K.nx) ? -1 : (K.bc_x == 5 ? K.sbc[x < 0 ? 0 : 1] : K.bc_x);
-    const int cy = (y >= 0 && y < K.ny) ? -1 : (K.bc_y == 5 ? K.sbc[y < 0 ? 2 : 3] : K.bc_y);
-    if (cy == 3) return K.sfeq[y < 0 ? 2 : 3][i];
-    if (cx == 3) return K.sfeq[x < 0 ? 0 : 1][i];
-    const int sx = cx == -1 ? x : map_index(x, K.nx, cx == 0 ? 0 : 1);
-    if (cy == 2) { // wall: the edge row plus its non-equilibrium correction (lambda copied)
-        const int side = y < 0 ? 0 : 1, sy = side ? K.ny - 1 : 0;
-        const R edge = __ldg(in + (size_t)i * K.plane + (size_t)sy * K.pitch + sx);
-        return i < NV ? edge + K.wall[((size_t)side * NV + i) * K.nx + sx] : edge;
-    }
-    int sy, ii = i;
-    if (cy == 4) {
-        sy = y < 0 ? -y - 1 : 2 * K.ny - 1 - y;
-        ii = mirror24(i);
-    } else {
-        sy = cy == -1 ? y : map_index(y, K.ny, cy == 0 ? 0 : 1);
-    }
-    return __ldg(in + (size_t)ii * K.plane + (size_t)sy * K.pitch + sx);
-}
-
 // rho, u_x, u_y and, if asked, T (FP64) at cell (x, y) of state `in`, boundary conditions
 // applied (Eqs. (5)-(7)). The sums go orbit by orbit: an orbit of speed c adds its sum s
 // to rho, c times its x and y differences to rho u, and (c^2 or 2 c^2) + eta^2 times s to
 // the energy moment m_4; 1/rho comes from an FP32 seed and two Newton steps.
-template <typename R, bool GEN = false>
+template <typename R>
 __device__ __forceinline__ void conserved_at(const Model<R>& K, const R* __restrict__ in, int x,
                                              int y, double& rho, double& ux, double& uy,
                                              double* T = nullptr)
 {
-    R gf[GEN ? NV : 1];
-    if constexpr (GEN) {
-#pragma unroll
-        for (int i = 0; i < NV; i++) gf[i] = fval(K, in, i, x, y);
-    }
     x = map_index(x, K.nx, K.bc_x == 0 ? 0 : 1);
     y = map_index(y, K.ny, K.bc_y == 0 ? 0 : 1);
     const R* p = in + (size_t)y * K.pitch + x;
-    // plane i of this cell: through the side rules, or straight from the mapped cell
-    auto ld = [&](int i) -> R {
-        if constexpr (GEN) return gf[i];
-        else return __ldg(p + (size_t)i * K.plane);
-    };
+    auto ld = [&](int i) -> R { return __ldg(p + (size_t)i * K.plane); };
     double r = 0.0, jx = 0.0, jy = 0.0, e = 0.0;
     if constexpr (sizeof(R) == 4) {
         // FP32 state: the same sums as double-floats on the FP32 pipes (error-free
@@ -447,197 +426,526 @@ __device__ __forceinline__ void block_tne(const R* Dk, bool active, double* part
     }
 }
 
+// ---- the step -----------------------------------------------------------------------
+// conserved moments of one cell from its butterflies g, then rho, u, T (Eqs. (5)-(7)); FP64
+struct Macro {
+    double rho, ux, uy, T;
+    bool hot, ok; // T > T_ig; rho, T > 0 and finite
+};
+__device__ __forceinline__ Macro recover24(const Model<double>& K, const double* f, const double* g)
+{
+    double P[6];
+#pragma unroll
+    for (int o = 0; o < 6; o++) P[o] = (o & 1) ? g[(o / 2) * 3 + 2] : ad(g[(o / 2) * 3], g[(o / 2) * 3 + 1]);
+    Macro m;
+    m.rho = ad(ad(ad(P[0], P[1]), ad(P[2], P[3])), ad(P[4], P[5]));
+    double jx = mu(K.cd[0], g[9]), jy = mu(K.cd[0], g[15]), e = mu(K.wod[0], P[0]);
+#pragma unroll
+    for (int o = 1; o < 6; o++) {
+        jx = fm(K.cd[o], g[9 + o], jx);
+        jy = fm(K.cd[o], g[15 + o], jy);
+        e = fm(K.wod[o], P[o], e);
+    }
+    const double q = lbk::recip64(m.rho);
+    m.ux = mu(jx, q);
+    m.uy = mu(jy, q);
+    m.T = mu(fm(e, q, -fm(m.ux, m.ux, mu(m.uy, m.uy))), K.inv_DI);
+    const long long rb = dbits(m.rho), tb = dbits(m.T), big = dbits(DBL_MAX);
+    m.ok = rb > 0 && rb <= big && tb > 0 && tb <= big;
+    m.hot = tb > dbits(K.T_ig);
+    return m;
+}
+// the same of an FP32 state: the sums exact double-floats on the FP32 pipes, carried into FP64
+__device__ __forceinline__ Macro recover24(const Model<float>& K, const float* f, const float*)
+{
+    using lbk::S1;
+    S1 r{0.f, 0.f}, jx{0.f, 0.f}, jy{0.f, 0.f}, e{0.f, 0.f};
+#pragma unroll
+    for (int o = 0; o < 6; o++) {
+        const float a = f[4 * o], b = f[4 * o + 1], c = f[4 * o + 2], d = f[4 * o + 3];
+        const S1 sac = lbk::s_sum(a, c), sbd = lbk::s_sum(b, d);
+        const S1 dac = lbk::s_sum(a, -c), dbd = lbk::s_sum(b, -d);
+        const S1 sum = lbk::s_add(sac, sbd);
+        const S1 gx = (o & 1) ? lbk::s_sub(dac, dbd) : dac, gy = (o & 1) ? lbk::s_add(dac, dbd) : dbd;
+        const S1 px = lbk::s_mul(gx, K.cdh[o], K.cdl[o]), py = lbk::s_mul(gy, K.cdh[o], K.cdl[o]);
+        const S1 pe = lbk::s_mul(sum, K.wdh[o], K.wdl[o]);
+        r = o ? lbk::s_add(r, sum) : sum;
+        jx = o ? lbk::s_add(jx, px) : px;
+        jy = o ? lbk::s_add(jy, py) : py;
+        e = o ? lbk::s_add(e, pe) : pe;
+    }
+    r = lbk::s_norm(r);
+    jx = lbk::s_norm(jx);
+    jy = lbk::s_norm(jy);
+    e = lbk::s_norm(e);
+    Macro m;
+    m.rho = lbk::df_to_f64_fast(r.hi, r.lo);
+    lbk::recover_one_f64_fast(r.hi, r.lo, m.rho, lbk::df_to_f64_fast(jx.hi, jx.lo),
+                              lbk::df_to_f64_fast(jy.hi, jy.lo), lbk::df_to_f64_fast(e.hi, e.lo), K.inv_DI,
+                              m.ux, m.uy, m.T);
+    const long long tb = dbits(m.T), big = dbits(DBL_MAX);
+    m.ok = r.hi > 0.f && r.hi <= FLT_MAX && fabsf(jx.hi) <= FLT_MAX && fabsf(jy.hi) <= FLT_MAX &&
+           fabsf(e.hi) <= FLT_MAX && tb > 0 && tb <= big;
+    m.hot = tb > dbits(K.T_ig);
+    return m;
+}
+
+// rows r of sector sct of B applied to x, columns j0.. only
+template <typename R>
+__device__ __forceinline__ R row_dot(const R* B, int sct, int r, int j0, const R* x)
+{
+    const int n = sec_n(sct), b0 = sec_b(sct) + r * n, p0 = sec_p(sct);
+    R acc = mu(B[b0 + j0], x[p0 + j0]);
+#pragma unroll
+    for (int j = 1; j < 9; j++)
+        if (j0 + j < n) acc = fm(B[b0 + j0 + j], x[p0 + j0 + j], acc);
+    return acc;
+}
+// the first moments of the sectors ee (m1, m4), oe (m2), eo (m3) are conserved
+__host__ __device__ constexpr int sec_cons(int s) { return s == 0 ? 2 : (s == 3 ? 0 : 1); }
+
+// velocity space from sector components whose butterfly scales B has folded in
+template <typename R>
+__device__ __forceinline__ void unfly(const R* g, R* f)
+{
+#pragma unroll
+    for (int o = 0; o < 6; o++) {
+        const int e0 = (o / 2) * 3;
+        if ((o & 1) == 0) {
+            f[4 * o] = ad(g[e0], g[9 + o]);
+            f[4 * o + 1] = ad(g[e0 + 1], g[15 + o]);
+            f[4 * o + 2] = ad(g[e0], -g[9 + o]);
+            f[4 * o + 3] = ad(g[e0 + 1], -g[15 + o]);
+        } else {
+            const R ep = ad(g[e0 + 2], g[21 + o / 2]), em = ad(g[e0 + 2], -g[21 + o / 2]);
+            const R xp = ad(g[9 + o], g[15 + o]), xm = ad(g[9 + o], -g[15 + o]);
+            f[4 * o] = ad(ep, xp);
+            f[4 * o + 1] = ad(em, -xm);
+            f[4 * o + 2] = ad(ep, -xp);
+            f[4 * o + 3] = ad(em, xm);
+        }
+    }
+}
+// M^-1 applied to w (sector order); CONS: the conserved entries are zero and left out
+template <bool CONS, typename R>
+__device__ __forceinline__ void inverse24(const Model<R>& K, const R* w, R* f)
+{
+    R g[NV];
+#pragma unroll
+    for (int sct = 0; sct < NSEC; sct++)
+#pragma unroll
+        for (int r = 0; r < 9; r++)
+            if (r < sec_n(sct)) g[sec_p(sct) + r] = row_dot(K.Bis, sct, r, CONS ? sec_cons(sct) : 0, w);
+    unfly(g, f);
+}
+
+// the products that f_hat^eq is made of
+template <typename R>
+struct Eq24 {
+    R m1, m2, m3, ux, uy, T, u2, Ta, Tb, A, B, pT, rIT, IT, C, G, H;
+};
+template <typename R>
+__device__ __forceinline__ Eq24<R> eq24(const Model<R>& K, R rho, R ux, R uy, R T)
+{
+    Eq24<R> e;
+    e.m1 = rho;
+    e.ux = ux;
+    e.uy = uy;
+    e.T = T;
+    e.m2 = mu(rho, ux);
+    e.m3 = mu(rho, uy);
+    const R ux2 = mu(ux, ux), uy2 = mu(uy, uy), I3 = mu(R(3), K.I_r);
+    e.u2 = ad(ux2, uy2);
+    e.Ta = ad(T, ux2);
+    e.Tb = ad(T, uy2);
+    e.A = fm(ad(K.DI_r, R(2)), T, e.u2);
+    e.B = fm(R(2), T, e.A);
+    e.pT = mu(rho, T);
+    e.IT = mu(K.I_r, T);
+    e.rIT = mu(rho, e.IT);
+    e.C = fm(e.u2, e.u2, mu(T, fm(ad(K.DI_r, R(10)), e.u2, mu(mu(R(4), ad(K.DI_r, R(4))), T))));
+    e.G = mu(e.IT, fm(ad(R(4), I3), T, e.u2));
+    e.H = fm(ad(R(2), I3), T, e.u2);
+    return e;
+}
+// f_hat^eq of moment k (0-based), and h - f_hat^eq with the last product inside an FMA
+template <typename R>
+__device__ __forceinline__ R minus_eq(const Eq24<R>& e, int k, R h)
+{
+    switch (k) {
+    case 4: return fm(-e.m1, e.Ta, h);
+    case 5: return fm(-e.m2, e.uy, h);
+    case 6: return fm(-e.m1, e.Tb, h);
+    case 7: return fm(-e.m2, e.A, h);
+    case 8: return fm(-e.m3, e.A, h);
+    case 9: return fm(-e.m2, fm(R(2), e.T, e.Ta), h);
+    case 10: return fm(-e.m3, e.Ta, h);
+    case 11: return fm(-e.m2, e.Tb, h);
+    case 12: return fm(-e.m3, fm(R(2), e.T, e.Tb), h);
+    case 13: return fm(-mu(e.m2, e.ux), e.B, fm(-e.pT, e.A, h));
+    case 14: return fm(-mu(e.m2, e.uy), e.B, h);
+    case 15: return fm(-mu(e.m3, e.uy), e.B, fm(-e.pT, e.A, h));
+    case 16: return fm(-e.rIT, e.Ta, h);
+    case 17: return fm(-mu(e.m2, e.uy), e.IT, h);
+    case 18: return fm(-e.rIT, e.Tb, h);
+    case 19: return fm(-e.rIT, e.H, h);
+    case 20: return fm(-e.m2, e.C, h);
+    case 21: return fm(-e.m3, e.C, h);
+    case 22: return fm(-e.m2, e.G, h);
+    default: return fm(-e.m3, e.G, h);
+    }
+}
+
+template <typename R>
+__device__ __forceinline__ R eq_moment(const Model<R>& K, const Eq24<R>& e, int k)
+{
+    return k == 0 ? e.m1 : k == 1 ? e.m2 : k == 2 ? e.m3 : k == 3 ? mu(e.m1, fm(K.DI_r, e.T, e.u2)) : -minus_eq(e, k, R(0));
+}
+
+// Per-warp TNE statistics of a tile row: row k of td (stride ld) holds Delta_{k+5} (k < TK), d
+// and d^2 of the block's cells; the lanes take one quantity each over the warp's cells in
+// `mask`, first the signed sums and minima, then the sums of |Delta| and maxima, and join them
+// to the launch's statistics acc [NQ]. FP64 terms add in FP64, FP32 terms as exact pairs.
+template <typename R>
+__device__ __forceinline__ void warp_tne24(const R* td, int ld, unsigned mask, double* acc)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll 1
+    for (int pass = 0; pass < 2; pass++) {
+        if (lane >= (pass ? TK : TK + 2)) continue;
+        const R* p = td + lane * ld;
+        double sum;
+        R m = R(0);
+        bool any = false;
+        if constexpr (sizeof(R) == 8) {
+            sum = 0.0;
+            const long long keep = pass ? 0x7fffffffffffffffll : -1ll, flip = pass ? -1ll : 0ll;
+            long long v = lbk::order64(DBL_MAX);
+            for (int j = 0; j < 32; j++) {
+                if (!(mask >> j & 1u)) continue;
+                sum += __longlong_as_double(__double_as_longlong(p[j]) & keep);
+                const long long k = lbk::order64(p[j]) ^ flip;
+                v = k < v ? k : v;
+            }
+            any = mask != 0;
+            m = lbk::unorder64(v ^ flip);
+        } else {
+            float s = 0.f, c = 0.f, v = FLT_MAX;
+            const float sign = pass ? -1.f : 1.f;
+            for (int j = 0; j < 32; j++) {
+                if (!(mask >> j & 1u)) continue;
+                const lbk::df t = lbk::two_sum(s, pass ? fabsf(p[j]) : p[j]);
+                s = t.hi;
+                c += t.lo;
+                v = fminf(v, sign * p[j]);
+            }
+            sum = (double)s + (double)c;
+            any = mask != 0;
+            m = sign * v;
+        }
+        const int qs = lane < TK ? (pass ? TK : 0) + lane : 3 * TK + lane; // d, d^2 at 4 TK, 4 TK + 1
+        acc[qs] += sum;
+        if (lane < TK && any) {
+            const int qm = (pass ? 3 * TK : 2 * TK) + lane;
+            acc[qm] = pass ? fmax(acc[qm], (double)m) : fmin(acc[qm], (double)m);
+        }
+    }
+}
+
+// Tiles of 32 x 8 (FP32) or 32 x 4 cells (2-D), 32 cells (1-D), one cell per thread.
+template <typename R, bool TWO_D>
+struct Tile24 {
+    static constexpr int TX = 32, TY = !TWO_D ? 1 : (sizeof(R) == 8 ? 4 : 8), TT = TX * TY;
+    static constexpr int HY = TWO_D ? 2 : 0, SW = TX + 4, SH = TY + 2 * HY, PS = SW * SH;
+    static constexpr int UW = TX + 2, UH = TWO_D ? TY + 2 : 1; // u of the tile and its rim
+    static constexpr size_t smem(bool tne)
+    {
+        return sizeof(R) * ((size_t)NP * PS + 2 * UW * UH) +
+               (tne ? sizeof(double) * (size_t)TY * NQ + sizeof(R) * (TK + 2) * (TT + 1) : 0);
+    }
+};
+
 // SRT: the single-relaxation-time fast path (all R_5..R_24 equal, no TNE due): with one
 // rate the moment-space relaxation is -R (f - M^-1 f_hat^eq) in velocity space (the SRT
 // form of Sec. V) and A_hat vanishes, so the forward transform of f is skipped and only
 // f^eq = M^-1 f_hat^eq is formed (it also feeds the chemical term of Eq. (24)).
-template <typename R, bool SRT, bool GEN>
-__global__ void __launch_bounds__(BT, sizeof(R) == 4 ? 3 : 1) step_kernel(const Model<R> K, const Args a)
+//
+// Each block walks tiles (grid-stride loop): the 25 planes of the tile and its two-cell halo
+// are staged in shared memory by asynchronous copies, all in flight together; rho, u, T of the
+// own cells and u of the rim are recovered; the cells are updated from registers and shared
+// memory.
+template <typename R, bool SRT, bool TWO_D, bool TNE>
+__global__ void __launch_bounds__((Tile24<R, TWO_D>::TT), (TWO_D ? 2 : 1))
+    step_kernel(const __grid_constant__ Model<R> K, const __grid_constant__ Args a)
 {
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const bool active = x < K.nx && y < K.ny;
-    const int64_t step = a.ctr->step;
-    const bool do_tne = !SRT && a.tne_every > 0 && (step % a.tne_every) == 0;
+    using C = Tile24<R, TWO_D>;
+    constexpr int TX = C::TX, TY = C::TY, TT = C::TT, SW = C::SW, SH = C::SH, PS = C::PS, HY = C::HY,
+                  UW = C::UW, UH = C::UH;
+    extern __shared__ __align__(16) unsigned char smem[];
+    R* sf = reinterpret_cast<R*>(smem);                        // [25][SH][SW]
+    R* su = sf + NP * PS;                                      // u_x, u_y  [2][UH][UW]
+    double* acc = reinterpret_cast<double*>(su + 2 * UH * UW); // the launch's statistics [TY][NQ]
+    R* td = reinterpret_cast<R*>(acc + TY * NQ);               // [TK + 2][TT + 1]
+
+    const int t = threadIdx.x, lx = t & 31, ly = t >> 5; // a warp is a row of the tile
     const R* __restrict__ in = static_cast<const R*>(a.in);
     R* __restrict__ out = static_cast<R*>(a.out);
-    R Dk[TK];
-#pragma unroll
-    for (int k = 0; k < TK; k++) Dk[k] = R(0);
-    bool bad = false;
+    const bool tne = TNE && a.tne_every > 0;
+    const int64_t step = tne ? a.ctr->step : 0;
+    const bool do_tne = tne && step % a.tne_every == 0;
+    if (do_tne)
+        for (int i = lx; i < NQ; i += 32) acc[ly * NQ + i] = tkind(i) == 0 ? 0.0 : (tkind(i) == 1 ? DBL_MAX : -DBL_MAX);
+    int bad = 0;
 
-    // 1. conserved sums and macros in FP64 (Eqs. (5)-(7)) of the block's cells and a
-    //    one-cell rim (the central differences of u need them), each computed once
-    __shared__ double s_rho[MAC_CELLS], s_ux[MAC_CELLS], s_uy[MAC_CELLS], s_T[MAC_CELLS];
-    {
-        const int bw = blockDim.x + 2, bh = K.ny > 1 ? blockDim.y + 2 : 1;
-        const int x0 = blockIdx.x * blockDim.x - 1, y0 = blockIdx.y * blockDim.y - (K.ny > 1);
-        for (int c = threadIdx.x + threadIdx.y * blockDim.x; c < bw * bh;
-             c += blockDim.x * blockDim.y) {
-            const int hx = c % bw, hy = c / bw;
-            conserved_at<R, GEN>(K, in, x0 + hx, y0 + hy, s_rho[c], s_ux[c], s_uy[c], &s_T[c]);
+    const int tiles_x = (K.nx + TX - 1) / TX, ntiles = tiles_x * ((K.ny + TY - 1) / TY);
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int x0 = (tile % tiles_x) * TX, y0 = (tile / tiles_x) * TY;
+        __syncthreads(); // the previous tile is done with shared memory
+        lbk::stage_tile<NP, SH, SW, TY, TWO_D>(in, sf, x0 - 2, y0 - HY, K.nx, K.ny, K.pitch, K.plane, K.sides,
+                                               K.sfeq, [](int p) { return mirror24(p); });
+        lbk::cp_commit();
+        lbk::cp_wait<0>();
+        __syncthreads();
+        if (TWO_D && K.wall && (y0 - HY < 0 || y0 + TY + HY > K.ny)) {
+            // walls: the staged ghost rows hold copies of the edge row; add its correction
+            for (int c = t; c < SW * SH; c += TT) {
+                const int r = c / SW, y = y0 - HY + r, side = y < 0 ? 0 : 1;
+                if ((y >= 0 && y < K.ny) || K.sides[2 + side] != 2) continue;
+                bool m_;
+                const int sx = lbk::source(x0 - 2 + c - r * SW, K.nx, K.sides, 0, m_);
+                if (sx < 0) continue; // a corner, never read
+                for (int i = 0; i < NV; i++) sf[i * PS + c] += K.wall[((size_t)side * NV + i) * K.nx + sx];
+            }
+            __syncthreads();
+        }
+        const int x = x0 + lx, y = y0 + ly;
+        const bool active = x < K.nx && y < K.ny;
+        const R* s0 = sf + (ly + HY) * SW + lx + 2;
+        R g[NV];
+        Macro m;
+        if (y < K.ny) { // whole warps past the last row have nothing to do
+            R f[NV];
+#pragma unroll
+            for (int i = 0; i < NV; i++) f[i] = s0[i * PS];
+            butterfly(f, g);
+            m = recover24(K, f, g);
+            if (active && !m.ok) bad = 1;
+            su[(ly + (TWO_D ? 1 : 0)) * UW + lx + 1] = to_fast<R>(m.ux);
+            su[(UH + ly + (TWO_D ? 1 : 0)) * UW + lx + 1] = to_fast<R>(m.uy);
+        }
+        if (!SRT) { // u of the rim; the row past the grid is one of a ragged tile's own
+            const int rows = TWO_D ? 2 * UW : 0, rim = rows + 2 * TY;
+            for (int c = t; c < rim || (TWO_D && y0 + TY > K.ny && c < rim + TX); c += TT) {
+                int rx, ry;
+                if (c < rows) rx = c % UW, ry = c < UW ? 0 : UH - 1;
+                else if (c < rim) rx = (c & 1) ? UW - 1 : 0, ry = (TWO_D ? 1 : 0) + (c - rows) / 2;
+                else rx = 1 + c - rim, ry = K.ny - y0 + 1;
+                const R* sr = sf + (ry + (TWO_D ? 1 : 0)) * SW + rx + 1;
+                R f[NV], h[NV];
+#pragma unroll
+                for (int i = 0; i < NV; i++) f[i] = sr[i * PS];
+                butterfly(f, h);
+                const Macro r = recover24(K, f, h);
+                su[ry * UW + rx] = to_fast<R>(r.ux);
+                su[(UH + ry) * UW + rx] = to_fast<R>(r.uy);
+            }
         }
         __syncthreads();
-    }
-    if (active) {
-        const size_t g = (size_t)y * K.pitch + x;
-        R f[NV];
-#pragma unroll
-        for (int i = 0; i < NV; i++) f[i] = __ldg(in + (size_t)i * K.plane + g);
-        const R lam0 = __ldg(in + (size_t)NV * K.plane + g);
+        if (y >= K.ny) continue;
 
-        const int bw = blockDim.x + 2, two = K.ny > 1;
-        const int c0 = (threadIdx.y + two) * bw + threadIdx.x + 1;
-        const double rho = s_rho[c0], ux = s_ux[c0], uy = s_uy[c0];
-        const double T = s_T[c0];
-        bad = !(rho > 0.0) || !(T > 0.0) || !isfinite(rho) || !isfinite(T);
-
-        const double pT = rho * T;
-
-        // 2. rho, u, T were recovered in FP64; the bulk from here on runs in R, including
-        //    the velocity gradients (second-order central differences)
-        const R rr = to_r<R>(rho), uxr = to_r<R>(ux), uyr = to_r<R>(uy), Tr = to_r<R>(T);
-        const R Ir = K.I_r;
-        const R gxx = (to_r<R>(s_ux[c0 + 1]) - to_r<R>(s_ux[c0 - 1])) * K.hdx_r;
-        const R gyx = (to_r<R>(s_uy[c0 + 1]) - to_r<R>(s_uy[c0 - 1])) * K.hdx_r;
-        R gxy = R(0), gyy = R(0);
-        if (two) {
-            gxy = (to_r<R>(s_ux[c0 + bw]) - to_r<R>(s_ux[c0 - bw])) * K.hdy_r;
-            gyy = (to_r<R>(s_uy[c0 + bw]) - to_r<R>(s_uy[c0 - bw])) * K.hdy_r;
+        const R rr = to_fast<R>(m.rho), uxr = to_fast<R>(m.ux), uyr = to_fast<R>(m.uy), Tr = to_fast<R>(m.T);
+        const Eq24<R> e = eq24(K, rr, uxr, uyr, Tr);
+        const R lam0 = s0[NV * PS];
+        // reaction over dt with p and T frozen at t_n (Eq. (28), m = n = 1), in FP64
+        const bool hot = m.hot && lam0 != R(1);
+        const bool react = __any_sync(0xffffffffu, hot);
+        R dlam = R(0), chem = R(0);
+        if (react && hot) {
+            const double pT = mu(m.rho, m.T);
+            const double d = reaction_increment<double>((double)lam0, mu(K.omega1, pT), mu(K.omega2, pT), K.dt);
+            const double rT = lbk::recip64(m.T);
+            dlam = to_fast<R>(d);
+            chem = to_fast<R>(mu(mu(K.kchem, d), mu(rT, rT))); // Q lambda' / (I (D+I) T^2)
         }
-
-        // 3. moments (block form), equilibrium moments, non-equilibrium parts
-        R q[NV];
-        feq24<R>(Ir, K.DI_r, rr, uxr, uyr, Tr, q);
-        if (!SRT) {
-            R gv[NV], h[NV];
-            butterfly(f, gv);
-            block_apply(K.Bf, gv, h);
+        R W[NV], fe[NV];
+        if constexpr (SRT) {
+            R w[NV];
 #pragma unroll
-            for (int p = 0; p < NV; p++)
-                if (mom_of(p) >= 4) Dk[mom_of(p) - 4] = h[p] - q[mom_of(p)];
-        }
-
-        // 4. relaxation with A_hat_8, A_hat_9 (Eqs. (3)-(4), sign as in Eq. (29))
-        R Om_hat[TK];
+            for (int p = 0; p < NV; p++) w[p] = eq_moment(K, e, mom_of(p));
+            inverse24<false>(K, w, fe);
 #pragma unroll
-        for (int k = 0; k < TK; k++) Om_hat[k] = -K.S[k + 4] * Dk[k];
-        if (!SRT) {
-            const R th = (gxx + gyy) / K.DI_r, pTr = rr * Tr, shear = gyx + gxy;
-            Om_hat[3] += pTr * K.A8c_r * (R(4) * uxr * (gxx - th) + R(2) * uyr * shear);
-            Om_hat[4] += pTr * K.A9c_r * (R(4) * uyr * (gyy - th) + R(2) * uxr * shear);
-        }
-
-        // 5. reaction over dt with p and T frozen at t_n (Eq. (28), m = n = 1)
-        double dlam = 0.0;
-        if (T > K.T_ig)
-            dlam = reaction_increment<double>((double)lam0, K.omega1 * pT, K.omega2 * pT, K.dt);
-        const double lrate = dlam / K.dt;
-
-        // 6. back-transform (block form), chemical term of Eq. (24) on f^eq = M^-1 f_hat^eq,
-        //    NND advection, forward Euler
-        const bool react = lrate != 0.0;
-        R Om[NV], fe[NV];
-        {
-            R w[NV], gv[NV];
-            if (!SRT) {
+            for (int i = 0; i < NV; i++) W[i] = mu(-K.S[4], sub(s0[i * PS], fe[i]));
+        } else {
+            // Delta of the non-conserved moments, in sector order
+            R w[NV];
 #pragma unroll
-                for (int p = 0; p < NV; p++) w[p] = mom_of(p) >= 4 ? Om_hat[mom_of(p) - 4] : R(0);
-                block_apply(K.Bi, w, gv);
-                unbutterfly(gv, Om);
+            for (int sct = 0; sct < NSEC; sct++)
+#pragma unroll
+                for (int r = 0; r < 9; r++)
+                    if (r < sec_n(sct)) {
+                        const int p = sec_p(sct) + r;
+                        w[p] = r < sec_cons(sct) ? R(0) : minus_eq(e, mom_of(p), row_dot(K.Bf, sct, r, 0, g));
+                    }
+            if (do_tne) {
+                R d2 = R(0);
+#pragma unroll
+                for (int p = 0; p < NV; p++)
+                    if (mom_of(p) >= 4) {
+                        td[(mom_of(p) - 4) * (TT + 1) + t] = w[p];
+                        d2 = fm(w[p], w[p], d2);
+                    }
+                td[TK * (TT + 1) + t] = sqrt(d2);
+                td[(TK + 1) * (TT + 1) + t] = d2;
+                const unsigned mask = __ballot_sync(0xffffffffu, active);
+                __syncwarp();
+                warp_tne24(td + ly * 32, TT + 1, mask, acc + ly * NQ);
             }
-            if (SRT || react) {
+            if (react) { // f^eq for the chemical term
+                if constexpr (sizeof(R) == 8) { // f - M^-1 Delta: no conserved entries, no f_hat^eq
+                    inverse24<true>(K, w, fe);
 #pragma unroll
-                for (int p = 0; p < NV; p++) w[p] = q[mom_of(p)];
-                block_apply(K.Bi, w, gv);
-                unbutterfly(gv, fe);
+                    for (int i = 0; i < NV; i++) fe[i] = sub(s0[i * PS], fe[i]);
+                } else { // M^-1 f_hat^eq: free of the rounding that Delta's cancellation brings in FP32
+                    R q[NV];
+#pragma unroll
+                    for (int p = 0; p < NV; p++) q[p] = eq_moment(K, e, mom_of(p));
+                    inverse24<false>(K, q, fe);
+                }
             }
-            if (SRT) {
+            // relaxation with A_hat_8, A_hat_9 (Eqs. (3)-(4), sign as in Eq. (29)) and back
 #pragma unroll
-                for (int i = 0; i < NV; i++) Om[i] = -K.S[4] * (f[i] - fe[i]);
+            for (int p = 0; p < NV; p++) w[p] = mom_of(p) >= 4 ? mu(-K.S[mom_of(p)], w[p]) : R(0);
+            {
+                const R* u0 = su + (ly + (TWO_D ? 1 : 0)) * UW + lx + 1;
+                const R* v0 = u0 + UH * UW;
+                const R gxx = mu(sub(u0[1], u0[-1]), K.hdx_r), gyx = mu(sub(v0[1], v0[-1]), K.hdx_r);
+                const R gxy = TWO_D ? mu(sub(u0[TWO_D ? UW : 0], u0[TWO_D ? -UW : 0]), K.hdy_r) : R(0);
+                const R gyy = TWO_D ? mu(sub(v0[TWO_D ? UW : 0], v0[TWO_D ? -UW : 0]), K.hdy_r) : R(0);
+                const R th = mu(TWO_D ? ad(gxx, gyy) : gxx, K.inv_DI_r), sh = mu(R(2), TWO_D ? ad(gyx, gxy) : gyx);
+                w[10] = fm(mu(e.pT, K.A8c_r), fm(uyr, sh, mu(mu(R(4), uxr), sub(gxx, th))), w[10]);  // m8
+                w[16] = fm(mu(e.pT, K.A9c_r), fm(uxr, sh, mu(mu(R(4), uyr), sub(gyy, th))), w[16]);  // m9
+            }
+            inverse24<true>(K, w, W);
+        }
+        if (react) {
+            // C_i = f_i^eq chem [-(1 + D) I T + I (v_i - u)^2 + eta_i^2] (Eq. (24)), the square
+            // multiplied out: per orbit a - b_x s_x - b_y s_y
+            const R base = fm(K.I_r, e.u2, mu(R(-3), e.IT)), i2 = mu(R(2), K.I_r);
+#pragma unroll
+            for (int o = 0; o < 6; o++) {
+                const R ao = mu(chem, ad(base, K.chem_o[o])), cc = mu(chem, mu(i2, K.c_r[o]));
+                const R bx = mu(cc, uxr), by = mu(cc, uyr);
+#pragma unroll
+                for (int j = 0; j < 4; j++) {
+                    const int i = 4 * o + j, sx = vsign_x(i), sy = vsign_y(i);
+                    R k = ao;
+                    if (sx) k = sx > 0 ? sub(k, bx) : ad(k, bx);
+                    if (sy) k = sy > 0 ? sub(k, by) : ad(k, by);
+                    W[i] = fm(fe[i], k, W[i]);
+                }
             }
         }
-        const R chem = react ? to_r<R>(K.Q * lrate / (K.I * K.DI * T * T)) : R(0);
-        const R base = R(-3) * Ir * Tr; // -(1 + D) I T
-        const int xm2 = map_index(x - 2, K.nx, K.bc_x == 0 ? 0 : 1);
-        const int xm1 = map_index(x - 1, K.nx, K.bc_x == 0 ? 0 : 1);
-        const int xp1 = map_index(x + 1, K.nx, K.bc_x == 0 ? 0 : 1);
-        const int xp2 = map_index(x + 2, K.nx, K.bc_x == 0 ? 0 : 1);
-        const int by = K.bc_y == 0 ? 0 : 1;
-        const size_t row = (size_t)y * K.pitch;
-        const size_t ym2 = (size_t)map_index(y - 2, K.ny, by) * K.pitch;
-        const size_t ym1 = (size_t)map_index(y - 1, K.ny, by) * K.pitch;
-        const size_t yp1 = (size_t)map_index(y + 1, K.ny, by) * K.pitch;
-        const size_t yp2 = (size_t)map_index(y + 2, K.ny, by) * K.pitch;
-        // stencil value of plane i at x + d (LX) or y + d (LY): the side rules for the
-        // per-side variant, the mapped offsets otherwise
-        auto LX = [&](int i, int d) -> R {
-            if constexpr (GEN) return fval(K, in, i, x + d, y);
-            const int xo = d == -2 ? xm2 : (d == -1 ? xm1 : (d == 1 ? xp1 : xp2));
-            return __ldg(in + (size_t)i * K.plane + row + xo);
+
+        // NND flux differences (upwind side fixed per velocity), Euler update; one rounding at
+        // the size of f
+        auto nnd = [&](const R* q, R q0, int d, bool neg) -> R {
+            const R l = q[-d], r = q[d];
+            return neg ? lbk::nnd3(sub(q0, l), sub(r, q0), sub(q[2 * d], r), true)
+                       : lbk::nnd3(sub(l, q[-2 * d]), sub(q0, l), sub(r, q0), false);
         };
-        auto LY = [&](int i, int d) -> R {
-            if constexpr (GEN) return fval(K, in, i, x, y + d);
-            const size_t yo = d == -2 ? ym2 : (d == -1 ? ym1 : (d == 1 ? yp1 : yp2));
-            return __ldg(in + (size_t)i * K.plane + yo + x);
+        auto nnd_by = [&](const R* q, R q0, int d, bool neg) -> R { // the side known at run time
+            const R* c = neg ? q + d : q;
+            const R c0 = neg ? *c : q0, l = c[-d];
+            return lbk::nnd3(sub(l, c[-2 * d]), sub(c0, l), sub(c[d], c0), neg);
         };
+        const size_t gi = (size_t)y * K.pitch + x;
 #pragma unroll
         for (int i = 0; i < NV; i++) {
-            R om = Om[i];
-            if (react) {
-                const R cx = K.vx[i] - uxr, cy = K.vy[i] - uyr;
-                om += fe[i] * chem * (base + Ir * (cx * cx + cy * cy) + K.eta2[i]);
-            }
-            const R* pl = in + (size_t)i * K.plane;
-            R adv = R(0);
-            if (vsign_x(i) > 0)
-                adv = K.vxs[i] * nnd_pos(LX(i, -2), LX(i, -1), f[i], LX(i, 1));
-            else if (vsign_x(i) < 0)
-                adv = K.vxs[i] * nnd_neg(LX(i, -1), f[i], LX(i, 1), LX(i, 2));
-            if (K.ny > 1) {
-                if (vsign_y(i) > 0)
-                    adv += K.vys[i] * nnd_pos(LY(i, -2), LY(i, -1), f[i], LY(i, 1));
-                else if (vsign_y(i) < 0)
-                    adv += K.vys[i] * nnd_neg(LY(i, -1), f[i], LY(i, 1), LY(i, 2));
-            }
-            out[(size_t)i * K.plane + g] = f[i] + K.dt_r * (om - adv);
+            const R f0 = s0[i * PS];
+            R w = W[i];
+            if (vsign_x(i)) w = fm(-K.vxs[i], nnd(s0 + i * PS, f0, 1, vsign_x(i) < 0), w);
+            if (TWO_D && vsign_y(i)) w = fm(-K.vys[i], nnd(s0 + i * PS, f0, SW, vsign_y(i) < 0), w);
+            if (active) out[(size_t)i * K.plane + gi] = fm(K.dt_r, w, f0);
         }
-
-        // 7. lambda: u . grad(lambda) with NND interface values, then the update
-        R la = R(0);
-        if (uxr > R(0))
-            la = uxr * K.inv_dx_r * nnd_pos(LX(NV, -2), LX(NV, -1), lam0, LX(NV, 1));
-        else if (uxr < R(0))
-            la = uxr * K.inv_dx_r * nnd_neg(LX(NV, -1), lam0, LX(NV, 1), LX(NV, 2));
-        if (K.ny > 1) {
-            if (uyr > R(0))
-                la += uyr * K.inv_dy_r * nnd_pos(LY(NV, -2), LY(NV, -1), lam0, LY(NV, 1));
-            else if (uyr < R(0))
-                la += uyr * K.inv_dy_r * nnd_neg(LY(NV, -1), lam0, LY(NV, 1), LY(NV, 2));
-        }
-        R ln = lam0 - K.dt_r * la + to_r<R>(dlam);
-        ln = ln < R(0) ? R(0) : (ln > R(1) ? R(1) : ln);
-        out[(size_t)NV * K.plane + g] = ln;
+        // lambda: u . grad(lambda) with NND interface values, then the update
+        const R* sl = s0 + NV * PS;
+        R la = fm(mu(mu(-K.dt_r, K.inv_dx_r), uxr), nnd_by(sl, lam0, 1, lbk::negative(uxr)), dlam);
+        if (TWO_D) la = fm(mu(mu(-K.dt_r, K.inv_dy_r), uyr), nnd_by(sl, lam0, SW, lbk::negative(uyr)), la);
+        if (active) out[(size_t)NV * K.plane + gi] = lbk::clamp01(ad(lam0, la));
     }
 
-    // TNE partials of the state read (all threads take part), status, step counter
-    const int t = threadIdx.x + threadIdx.y * blockDim.x;
-    const int b = blockIdx.x + blockIdx.y * gridDim.x, nb = gridDim.x * gridDim.y;
-    if (do_tne) block_tne(Dk, active, a.partials, nb, b);
+    // status, TNE partials, step counter: without TNE no block reads the counter, so block 0
+    // moves it on; with TNE the last block to finish does
     if (__syncthreads_or(bad) && t == 0) atomicOr(&a.ctr->status, 1);
-    __shared__ unsigned int s_last;
-    if (t == 0) s_last = (atomicAdd(&a.ctr->arrivals, 1u) == (unsigned)nb - 1) ? 1u : 0u;
-    __syncthreads();
-    if (s_last && t == 0) {
-        if (do_tne) {
-            a.ctr->hist_count += 1;
-            a.ctr->tne_step = step;
+    if (do_tne)
+        for (int q = t; q < NQ; q += TT) {
+            double v = acc[q];
+            for (int w = 1; w < TY; w++) v = tcomb(tkind(q), v, acc[w * NQ + q]);
+            a.partials[(size_t)q * gridDim.x + blockIdx.x] = v;
         }
-        a.ctr->tne_pending = do_tne ? 1 : 0;
-        a.ctr->step = step + 1;
-        a.ctr->arrivals = 0u;
+    if (!tne) {
+        if (blockIdx.x == 0 && t == 0) {
+            a.ctr->tne_pending = 0;
+            a.ctr->step += 1;
+        }
+    } else if (t == 0) {
+        if (atomicAdd(&a.ctr->arrivals, 1u) == gridDim.x - 1) {
+            if (do_tne) {
+                a.ctr->hist_count += 1;
+                a.ctr->tne_step = step;
+            }
+            a.ctr->tne_pending = do_tne ? 1 : 0;
+            a.ctr->step = step + 1;
+            a.ctr->arrivals = 0u;
+        }
     }
 }
+
+template <typename R, bool SRT, bool TWO_D, bool TNE>
+cudaError_t step_prepare()
+{
+    static cudaError_t done = cudaFuncSetAttribute(step_kernel<R, SRT, TWO_D, TNE>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                   (int)Tile24<R, TWO_D>::smem(TNE));
+    return done;
+}
+// blocks of a launch: all tiles, or as many as the SMs hold at a time
+template <typename R, bool SRT, bool TWO_D, bool TNE>
+int step_blocks(int nx, int ny, int sms)
+{
+    using C = Tile24<R, TWO_D>;
+    static int per_sm = -1;
+    if (per_sm < 0) {
+        if (step_prepare<R, SRT, TWO_D, TNE>() != cudaSuccess) return -1;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel<R, SRT, TWO_D, TNE>, C::TT,
+                                                          C::smem(TNE)) != cudaSuccess)
+            return -1;
+        if (per_sm < 1) per_sm = 1;
+    }
+    const int64_t tiles = (int64_t)((nx + C::TX - 1) / C::TX) * ((ny + C::TY - 1) / C::TY);
+    const int64_t g = (int64_t)per_sm * sms;
+    return (int)(tiles < g ? tiles : g);
+}
+template <typename R, bool SRT, bool TWO_D, bool TNE>
+cudaError_t step_launch(const Model<R>& K, const Args& a, int blocks, cudaStream_t s)
+{
+    using C = Tile24<R, TWO_D>;
+    const cudaError_t e = step_prepare<R, SRT, TWO_D, TNE>();
+    if (e != cudaSuccess) return e;
+    step_kernel<R, SRT, TWO_D, TNE><<<blocks, C::TT, C::smem(TNE), s>>>(K, a);
+    return cudaGetLastError();
+}
+// the step variant of a handle: CALL(R, SRT, TWO_D, TNE) of its precision, collision, shape and
+// records
+#define V24_VARIANT(CALL, f64, srt, two_d, tne)                                                    \
+    ((f64) ? ((two_d) ? ((srt) ? CALL(double, true, true, false)                                   \
+                         : (tne) ? CALL(double, false, true, true) : CALL(double, false, true, false)) \
+                      : ((srt) ? CALL(double, true, false, false)                                  \
+                         : (tne) ? CALL(double, false, false, true) : CALL(double, false, false, false))) \
+           : ((two_d) ? ((srt) ? CALL(float, true, true, false)                                    \
+                         : (tne) ? CALL(float, false, true, true) : CALL(float, false, true, false)) \
+                      : ((srt) ? CALL(float, true, false, false)                                   \
+                         : (tne) ? CALL(float, false, false, true) : CALL(float, false, false, false))))
 
 // TNE of a state on demand: Delta fields (optional) and block partials.
 template <typename R>
@@ -715,9 +1023,9 @@ __global__ void wall_kernel(const Model<R> K, const R* __restrict__ in, R* wall)
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= 2 * K.nx) return;
     const int side = t / K.nx, x = t % K.nx;
-    if (K.sbc[2 + side] != 2) return;
+    if (K.sides[2 + side] != 2) return;
     double rho, ux, uy, T;
-    conserved_at<R, false>(K, in, x, side ? K.ny - 1 : 0, rho, ux, uy, &T);
+    conserved_at(K, in, x, side ? K.ny - 1 : 0, rho, ux, uy, &T);
     double qw[NV], qf[NV];
     feq24<double>(K.I, K.DI, rho, K.wux[side], K.wuy[side], K.wT[side], qw);
     feq24<double>(K.I, K.DI, rho, ux, uy, T, qf);
@@ -730,24 +1038,24 @@ __global__ void wall_kernel(const Model<R> K, const R* __restrict__ in, R* wall)
     }
 }
 
+// f = M^-1 f_hat^eq in block form, FP64 (162 multiply-adds of the transform, not 576)
 template <typename R>
-__global__ void init_kernel(const Model<R> K, const double* rho, const double* ux,
+__global__ void init_kernel(const __grid_constant__ Model<double> K, const double* rho, const double* ux,
                             const double* uy, const double* T, const double* lam, R* state)
 {
     const int64_t n = (int64_t)K.nx * K.ny;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < n;
          c += (int64_t)gridDim.x * blockDim.x) {
         const int x = (int)(c % K.nx), y = (int)(c / K.nx);
-        double q[NV];
-        feq24<double>(K.I, K.DI, rho[c], ux[c], uy[c], T[c], q);
+        const double t = T[c];
+        const Eq24<double> e = eq24(K, rho[c], ux[c], uy[c], t);
+        double w[NV], f[NV];
+#pragma unroll
+        for (int p = 0; p < NV; p++) w[p] = eq_moment(K, e, mom_of(p));
+        inverse24<false>(K, w, f);
         const size_t g = (size_t)y * K.pitch + x;
 #pragma unroll
-        for (int i = 0; i < NV; i++) {
-            double s = 0.0;
-#pragma unroll
-            for (int k = 0; k < NV; k++) s = fma(K.Minvd[i * NV + k], q[k], s);
-            state[(size_t)i * K.plane + g] = (R)s;
-        }
+        for (int i = 0; i < NV; i++) state[(size_t)i * K.plane + g] = (R)f[i];
         state[(size_t)NV * K.plane + g] = lam ? (R)lam[c] : R(0);
     }
 }
@@ -917,9 +1225,19 @@ void fill_model(const lbkm24_params& p, const double* Bf, const double* Bi, cons
 {
     memset(K, 0, sizeof(*K));
     for (int sd = 0; sd < 4; sd++) {
-        K->sbc[sd] = sbc[sd];
+        const int dir = sd < 2 ? p.bc_x : p.bc_y;
+        K->sides[sd] = dir == LBKM_BC_SIDES ? sbc[sd] : dir;
         for (int i = 0; i < NP; i++) K->sfeq[sd][i] = (R)sfeq[sd][i];
     }
+    for (int sct = 0; sct < NSEC; sct++)
+        for (int r = 0; r < sec_n(sct); r++) {
+            // orbit parity of component r: ee (sx, sy, e) per group, oe and eo one per orbit
+            const bool diag = sct == 0 ? r % 3 == 2 : (sct == 3 ? true : r & 1);
+            for (int j = 0; j < sec_n(sct); j++) {
+                const int k = sec_b(sct) + r * sec_n(sct) + j;
+                K->Bis[k] = (R)(Bi[k] * (diag ? 0.25 : 0.5));
+            }
+        }
     for (int k = 0; k < NB; k++) {
         K->Bf[k] = (R)Bf[k];
         K->Bi[k] = (R)Bi[k];
@@ -945,6 +1263,13 @@ void fill_model(const lbkm24_params& p, const double* Bf, const double* Bi, cons
     }
     K->I = 2.0 / (p.gamma - 1.0) - 2.0;
     K->DI = 2.0 + K->I;
+    K->kchem = p.Q / (p.dt * K->I * K->DI);
+    K->inv_DI_r = (R)(1.0 / K->DI);
+    for (int o = 0; o < 6; o++) {
+        const double c = p.v[o / 2], et = p.eta[o / 2];
+        K->c_r[o] = (R)c;
+        K->chem_o[o] = (R)(K->I * c * c * ((o & 1) ? 2.0 : 1.0) + et * et);
+    }
     K->inv_DI = 1.0 / K->DI;
     K->Q = p.Q;
     K->omega1 = p.omega1;
@@ -992,8 +1317,9 @@ struct lbkm24 {
     void* buf[2];
     int cur;
     double* partials;
-    int nblocks;
+    int nblocks;       // of tne_kernel
     dim3 grid, block;
+    int sblocks;       // of a step
     DevCounters* ctr;
     Record* hist;
     Record* tne_out;
@@ -1038,7 +1364,6 @@ cudaError_t launch_one_step(const lbkm24* h, int from, cudaStream_t st)
     a.hist_cap = h->p.tne_capacity;
     a.tne_every = h->p.tne_every;
     a.area = h->p.dx * h->p.dy;
-    const bool gen = h->p.bc_x == LBKM_BC_SIDES || h->p.bc_y == LBKM_BC_SIDES;
     if (h->has_wall) {
         const int g = (2 * h->p.nx + 127) / 128;
         if (h->p.precision == LBKM_F64)
@@ -1048,21 +1373,13 @@ cudaError_t launch_one_step(const lbkm24* h, int from, cudaStream_t st)
         const cudaError_t we = cudaGetLastError();
         if (we != cudaSuccess) return we;
     }
-#define V24_LAUNCH(R_, KK)                                                                   \
-    do {                                                                                     \
-        if (h->srt && gen) step_kernel<R_, true, true><<<h->grid, h->block, 0, st>>>(KK, a); \
-        else if (h->srt) step_kernel<R_, true, false><<<h->grid, h->block, 0, st>>>(KK, a);  \
-        else if (gen) step_kernel<R_, false, true><<<h->grid, h->block, 0, st>>>(KK, a);     \
-        else step_kernel<R_, false, false><<<h->grid, h->block, 0, st>>>(KK, a);             \
-    } while (0)
-    if (h->p.precision == LBKM_F64)
-        V24_LAUNCH(double, h->Kd);
-    else
-        V24_LAUNCH(float, h->Kf);
+    const bool f64 = h->p.precision == LBKM_F64;
+#define V24_LAUNCH(R_, SRT_, D2_, TNE_) \
+    step_launch<R_, SRT_, D2_, TNE_>(*static_cast<const Model<R_>*>(f64 ? (const void*)&h->Kd : &h->Kf), a, h->sblocks, st)
+    cudaError_t e = V24_VARIANT(V24_LAUNCH, f64, h->srt, h->p.ny > 1, h->p.tne_every > 0);
 #undef V24_LAUNCH
-    cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && h->p.tne_every > 0) {
-        finish_kernel<<<NQ, 256, 0, st>>>(h->partials, h->nblocks, h->hist, h->p.tne_capacity,
+        finish_kernel<<<NQ, 256, 0, st>>>(h->partials, h->sblocks, h->hist, h->p.tne_capacity,
                                           h->ctr, nullptr, a.area);
         e = cudaGetLastError();
     }
@@ -1247,8 +1564,7 @@ lbkm_status lbkm24_create(const lbkm24_params* pin, void* cuda_stream, lbkm24_t*
         h->Kd.wuy[w] = h->Kf.wuy[w] = p.side_uy[2 + w];
         h->Kd.wT[w] = h->Kf.wT[w] = p.side_T[2 + w];
     }
-    // 1-D grids too short to give every SM a block of 128 cells run blocks of one warp:
-    // the step is latency-bound there, and more SMs each take fewer cells
+    // (the TNE of a state on demand: short 1-D grids in blocks of one warp, for more SMs)
     const bool narrow = p.ny == 1 && (p.nx + BT - 1) / BT < 2 * sm_count();
     h->block = p.ny > 1 ? dim3(32, BT / 32) : dim3(narrow ? 32 : BT, 1);
     h->grid = dim3((p.nx + h->block.x - 1) / h->block.x, (p.ny + h->block.y - 1) / h->block.y);
@@ -1259,10 +1575,16 @@ lbkm_status lbkm24_create(const lbkm24_params* pin, void* cuda_stream, lbkm24_t*
                     what, cudaGetErrorString(ce));
     };
     cudaError_t ce;
+    const int sms = sm_count();
+#define V24_BLOCKS(R_, SRT_, D2_, TNE_) step_blocks<R_, SRT_, D2_, TNE_>(p.nx, p.ny, sms)
+    h->sblocks = V24_VARIANT(V24_BLOCKS, p.precision == LBKM_F64, h->srt, p.ny > 1, p.tne_every > 0);
+#undef V24_BLOCKS
+    if (h->sblocks < 1) return bail(cudaGetLastError(), "step kernel");
     const size_t sb = (size_t)NP * h->plane_elems * h->elem;
     for (int k = 0; k < 2; k++)
         if ((ce = cudaMalloc(&h->buf[k], sb)) != cudaSuccess) return bail(ce, "state");
-    if ((ce = cudaMalloc((void**)&h->partials, sizeof(double) * NQ * h->nblocks)) != cudaSuccess)
+    if ((ce = cudaMalloc((void**)&h->partials, sizeof(double) * NQ * (h->nblocks > h->sblocks ? h->nblocks : h->sblocks))) !=
+        cudaSuccess)
         return bail(ce, "partials");
     if (h->has_wall) {
         const size_t wb = sizeof(double) * 2 * NV * (size_t)p.nx;
@@ -1329,7 +1651,7 @@ lbkm_status lbkm24_init_fields(lbkm24_t h, const double* rho, const double* ux, 
         init_kernel<double><<<g, 256, 0, h->stream>>>(h->Kd, dev[0], dev[1], dev[2], dev[3],
                                                       dev[4], (double*)h->buf[0]);
     else
-        init_kernel<float><<<g, 256, 0, h->stream>>>(h->Kf, dev[0], dev[1], dev[2], dev[3],
+        init_kernel<float><<<g, 256, 0, h->stream>>>(h->Kd, dev[0], dev[1], dev[2], dev[3],
                                                      dev[4], (float*)h->buf[0]);
     TRY24(h, cudaGetLastError());
     h->cur = 0;

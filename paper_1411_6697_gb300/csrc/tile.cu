@@ -98,29 +98,8 @@ __global__ void __launch_bounds__(Tile<R>::TT, sizeof(R) == 8 ? 2 : 4)
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int x0 = (tile % tiles_x) * TX, y0 = (tile / tiles_x) * TY;
         __syncthreads(); // the previous tile is done with shared memory
-        // stage: a warp copies a row of all planes, lane c the columns c (and 32 + c) of the
-        // staged SW, all copies in flight together; Dirichlet ghosts are stored
-        {
-            bool m_;
-            const int c0 = source(x0 - 2 + lx, nx, K.sbc, 0, m_), c1 = source(x0 + 30 + lx, nx, K.sbc, 0, m_);
-            for (int r = ly; r < SH; r += TW) {
-                bool mir;
-                const int gy = source(y0 - 2 + r, ny, K.sbc, 2, mir);
-                R* dst = sf + r * SW + lx;
-                const R* src = in + (int64_t)(gy < 0 ? 0 : gy) * pitch;
-#pragma unroll
-                for (int p = 0; p < NPLANE; p++) {
-                    const R* sp = src + (mir ? mirror_plane(p) : p) * plane;
-                    const int g0 = gy < 0 ? gy : c0, g1 = gy < 0 ? gy : c1; // a Dirichlet row: all of it
-                    if (g0 >= 0) cp1(dst + p * PS, sp + g0);
-                    else dst[p * PS] = K.sfeq[-1 - g0][p];
-                    if (lx < SW - 32) {
-                        if (g1 >= 0) cp1(dst + p * PS + 32, sp + g1);
-                        else dst[p * PS + 32] = K.sfeq[-1 - g1][p];
-                    }
-                }
-            }
-        }
+        stage_tile<NPLANE, SH, SW, TW, true>(in, sf, x0 - 2, y0 - 2, nx, ny, pitch, plane, K.sbc, K.sfeq,
+                                             [](int p) { return mirror_plane(p); });
         cp_commit();
         cp_wait<0>();
         __syncthreads();
