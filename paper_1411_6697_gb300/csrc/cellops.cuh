@@ -444,8 +444,8 @@ __device__ __forceinline__ void recover64(const ModelConst<double>& K, const Fly
                                           double& uy2, double& u2, double& T, bool& ok)
 {
     m1 = (b.P0 + b.P2) + (b.e1 + b.e3);
-    m2 = fm(K.cd[3], b.ax3, fm(K.cd[1], b.ax1, fm(K.cd[2], b.ax2, mu(K.cd[0], b.ax0))));
-    m3 = fm(K.cd[3], b.ay3, fm(K.cd[1], b.ay1, fm(K.cd[2], b.ay2, mu(K.cd[0], b.ay0))));
+    m2 = fm(K.cd[3], b.ax3, fm(K.cd[2], b.ax2, fm(K.cd[1], b.ax1, mu(K.cd[0], b.ax0))));
+    m3 = fm(K.cd[3], b.ay3, fm(K.cd[2], b.ay2, fm(K.cd[1], b.ay1, mu(K.cd[0], b.ay0))));
     const double m4 = fm(K.wd[3], b.e3, fm(K.wd[1], b.e1, fm(K.wd[2], b.P2, mu(K.wd[0], b.P0))));
     const double q = recip64(m1);
     ux = mu(m2, q);
