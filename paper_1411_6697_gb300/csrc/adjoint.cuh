@@ -1,8 +1,29 @@
-// The objective of the discrete adjoint without its derivative (adjoint.cu).
+// The discrete adjoint's reverse sweep and the objective without its derivative (adjoint.cu).
 #pragma once
 #include "kernels.cuh"
 
 namespace lbk {
+
+// How the reverse sweep cuts a grid: blocks of `threads` cells, of which the middle
+// threads - 4 steps - 4 are the block's own, `steps` reverse steps per launch.
+struct AdjPlan {
+    int threads, steps, grid;
+};
+AdjPlan adj_plan(int nx);
+
+struct AdjReverse {
+    const double* state; // the last state to reverse, 17 planes with the handle's pitch
+    int64_t stride;      // elements from a state back to the one before
+    int steps;           // states to reverse, 1 .. plan.steps
+    const double *fb1, *lb1; // dJ/df [16][nx] and dJ/dlambda [nx] after the last step
+    double *fb0, *lb0;       // the same before the first
+    double* pacc;        // [ADJ_NPAR][plan.grid] per-block parameter accumulators
+    double* jacc;        // [plan.grid] per-block objective accumulators
+    double jw;           // w_tne dx dt for the objective value
+};
+// tne_w: w_tne dx dt, Delta_b += 2 tne_w Delta
+cudaError_t launch_adj_reverse(const ModelConst<double>& K, const AdjReverse& a, const AdjPlan& p,
+                               double tne_w, cudaStream_t s);
 
 // Adds w_tne dx dt sum_x d^2 of the FP64 state a.f (d^2 = sum_{k=5..16} Delta_k^2,
 // Sec. VI, Eq. (91); rho, u, T recovered in the kernel) to the per-block accumulators

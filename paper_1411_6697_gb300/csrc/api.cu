@@ -1058,7 +1058,9 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
     const int64_t N = ob->steps;
     const int C = ob->checkpoint_every;
     const int64_t nck = (N + C - 1) / C;
-    const int G = adj_grid(nx);
+    const int Gs = adj_grid(nx); // blocks of the cell-wise kernels
+    const AdjPlan rplan = adj_plan(nx);
+    const int G = rplan.grid;
     // With an FP32 handle the forward run is the FP32 step and keeps FP32 checkpoints;
     // each segment is recomputed in FP64 from its checkpoint widened to FP64 and reversed
     // in FP64, so the derivative is taken along FP64 segments restarted from the FP32
@@ -1069,50 +1071,35 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
     const size_t SBf = h->state_bytes_dev;                  // forward states, checkpoints
     const size_t SBd = (size_t)NPLANE * h->plane_elems * 8; // FP64 segment states
     char *ck = nullptr, *seg = nullptr;
-    double *work = nullptr, *mats = nullptr;
+    double* work = nullptr;
     DevCounters* sctr = nullptr;
     auto cleanup = [&]() {
         cudaStreamSynchronize(h->stream);
         dfree(h, ck);
         dfree(h, seg);
         dfree(h, work);
-        dfree(h, mats);
         dfree(h, sctr);
     };
-    // work: mac 4n, mb 16n, loc 6n, gb 2n, fbA/fbB 32n, lbA/lbB 2n, rho_t n, drho0 n,
-    //       cw 85n, pacc NPAR*G, jtne G, jmis G
-    const size_t nwork = (size_t)nx * (4 + 16 + 6 + 2 + 32 + 2 + 1 + 1 + 85) + (size_t)(ADJ_NPAR + 2) * G;
+    // work: fbA/fbB 32n, lbA/lbB 2n, rho_t n, drho0 n, pacc NPAR*G, jtne G, jmis Gs
+    const size_t nwork = (size_t)nx * (32 + 2 + 1 + 1) + (size_t)(ADJ_NPAR + 1) * G + Gs;
     cudaError_t e = dmalloc(h, &ck, SBf * nck);
     if (e == cudaSuccess) e = dmalloc(h, &seg, SBd * (size_t)(C + 1));
     if (e == cudaSuccess) e = dmalloc(h, &work, sizeof(double) * nwork);
-    if (e == cudaSuccess) e = dmalloc(h, &mats, sizeof(double) * 16);
     if (e == cudaSuccess) e = dmalloc(h, &sctr, sizeof(DevCounters));
     if (e != cudaSuccess) {
         cleanup();
         return fail(h, e == cudaErrorMemoryAllocation ? LBKM_ENOMEM : LBKM_ECUDA,
                     "lbkm_grad allocation: %s", cudaGetErrorString(e));
     }
-    double* mac = work;
-    double* mb = mac + 4 * (size_t)nx;
-    double* loc = mb + 16 * (size_t)nx;
-    double* gb = loc + 6 * (size_t)nx;
-    double* fbA = gb + 2 * (size_t)nx;
+    double* fbA = work;
     double* fbB = fbA + 16 * (size_t)nx;
     double* lbA = fbB + 16 * (size_t)nx;
     double* lbB = lbA + nx;
     double* rho_t = lbB + nx;
     double* drho0 = rho_t + nx;
-    double* cw = drho0 + nx;
-    double* pacc = cw + 85 * (size_t)nx;
+    double* pacc = drho0 + nx;
     double* jtne = pacc + (size_t)ADJ_NPAR * G;
     double* jmis = jtne + G;
-    std::vector<double> hm(16); // x-velocities of the 16 f_i
-    {
-        static const int ax[4] = {1, 0, -1, 0}, dg[4] = {1, -1, -1, 1};
-        for (int o = 0; o < 4; o++)
-            for (int q = 0; q < 4; q++)
-                hm[4 * o + q] = h->hm.c[o] * (h->p.orbit_kind[o] == 0 ? ax[q] : dg[q]);
-    }
     cudaStream_t st = h->stream;
     auto S = [&](int64_t k) { return seg + (size_t)k * SBd; };
     auto K_ = [&](int64_t k) { return ck + (size_t)k * SBf; };
@@ -1124,9 +1111,8 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
             return fail(h, LBKM_ECUDA, "lbkm_grad: %s: %s", #call, cudaGetErrorString(e));   \
         }                                                                                     \
     } while (0)
-    GT(cudaMemcpyAsync(mats, hm.data(), sizeof(double) * hm.size(), cudaMemcpyHostToDevice, st));
     GT(cudaMemcpyAsync(rho_t, ob->rho_target, sizeof(double) * nx, cudaMemcpyHostToDevice, st));
-    GT(cudaMemsetAsync(pacc, 0, sizeof(double) * (ADJ_NPAR + 2) * G, st));
+    GT(cudaMemsetAsync(pacc, 0, sizeof(double) * ((size_t)(ADJ_NPAR + 1) * G + Gs), st));
     GT(cudaMemsetAsync(sctr, 0, sizeof(DevCounters), st));
     GT(cudaMemcpyAsync(K_(0), h->buf[h->cur], SBf, cudaMemcpyDeviceToDevice, st));
     LineArgs sl = line_args(h, 0, 1);
@@ -1135,49 +1121,43 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
     LineArgs sd = sl; // the FP64 steps of the recomputed segments: every state is kept
     const LinePlan dplan = f32 ? line_plan(0, nx) : h->line;
     sd.out_stride = (int64_t)(SBd / sizeof(double));
-    // forward run in the handle's precision, keeping a state every C steps
+    // forward run in the handle's precision, keeping a state every C steps, up to the last of
+    // them: the segment from there is formed below with all its states, the final one included
     const void* fwd = K_(0);
     int at = 0; // which of S(0), S(1) the run writes next
-    for (int64_t n = 0; n < N;) {
-        const int64_t next = (n / C + 1) * C < N ? (n / C + 1) * C : N;
+    for (int64_t n = 0, last = (nck - 1) * C; n < last;) {
+        const int64_t next = (n / C + 1) * C;
         sl.nsteps = (int)(next - n < h->line.steps ? next - n : h->line.steps);
         n += sl.nsteps;
         sl.in = fwd;
-        sl.out = n == next && n < N ? K_(n / C) : S(at);
+        sl.out = n == next ? K_(n / C) : S(at);
         GT(launch_line(h->precision, h->recovery, model_ptr(h), h->line, sl, st));
         fwd = sl.out;
         at ^= 1;
     }
     AdjArgs a;
     memset(&a, 0, sizeof(a));
-    a.mac = mac;
-    a.mb = mb;
-    a.loc = loc;
-    a.gb = gb;
-    a.cw = cw;
-    a.pacc = pacc;
-    a.vx = mats;
-    a.tne_w = ob->w_tne * h->p.dx * h->p.dt;
-    a.jw = a.tne_w;
-    // FP64 forward: seed with the mismatch of the final state now; FP32 forward: once the
-    // last segment has been recomputed in FP64
+    AdjReverse rv;
+    memset(&rv, 0, sizeof(rv));
+    rv.stride = (int64_t)(SBd / sizeof(double));
+    rv.pacc = pacc;
+    rv.jacc = jtne;
+    rv.jw = ob->w_tne * h->p.dx * h->p.dt;
+    // the sweep starts from the mismatch of the final state, once the last segment is formed
     a.fb0 = fbA;
     a.lb0 = lbA;
     auto seed = [&](const void* final_state) -> cudaError_t {
         a.f = static_cast<const double*>(final_state);
         a.jacc = jmis;
-        const cudaError_t se = launch_adj_seed(h->Kd, a, rho_t, ob->w_mismatch, G, st);
-        a.jacc = jtne;
-        return se;
+        return launch_adj_seed(h->Kd, a, rho_t, ob->w_mismatch, Gs, st);
     };
-    if (!f32) GT(seed(fwd));
     double *fc = fbA, *fn = fbB, *lc = lbA, *ln = lbB;
     for (int64_t sg = nck - 1; sg >= 0; sg--) {
         const int64_t n0 = sg * C, n1 = (n0 + C < N) ? n0 + C : N;
-        const bool last = f32 && sg == nck - 1; // recompute through the final state
+        const bool last = sg == nck - 1; // through the final state
         if (f32)
             GT(launch_adj_widen(reinterpret_cast<const float*>(K_(sg)), reinterpret_cast<double*>(S(0)),
-                                (size_t)NPLANE * h->plane_elems, G, st));
+                                (size_t)NPLANE * h->plane_elems, Gs, st));
         else
             GT(cudaMemcpyAsync(S(0), K_(sg), SBf, cudaMemcpyDeviceToDevice, st));
         for (int64_t n = n0, end = last ? n1 : n1 - 1; n < end; n += sd.nsteps) {
@@ -1187,16 +1167,14 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
             GT(launch_line(0, 0, &h->Kd, dplan, sd, st));
         }
         if (last) GT(seed(S(n1 - n0)));
-        for (int64_t n = n1 - 1; n >= n0; n--) {
-            const double* state = reinterpret_cast<const double*>(S(n - n0));
-            GT(launch_macros(0, h->Kd, state, mac, mac + nx, mac + 2 * (size_t)nx,
-                             mac + 3 * (size_t)nx, nullptr, nullptr, st));
-            a.f = state;
-            a.fb1 = fc;
-            a.lb1 = lc;
-            a.fb0 = fn;
-            a.lb0 = ln;
-            GT(launch_adj_step(h->Kd, a, G, st));
+        for (int64_t n = n1; n > n0; n -= rv.steps) { // the states n - 1, n - 2, ...
+            rv.steps = (int)(n - n0 < rplan.steps ? n - n0 : rplan.steps);
+            rv.state = reinterpret_cast<const double*>(S(n - 1 - n0));
+            rv.fb1 = fc;
+            rv.lb1 = lc;
+            rv.fb0 = fn;
+            rv.lb0 = ln;
+            GT(launch_adj_reverse(h->Kd, rv, rplan, rv.jw, st));
             std::swap(fc, fn);
             std::swap(lc, ln);
         }
@@ -1205,8 +1183,8 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
     // first segment's recomputation left in S(0))
     a.f = reinterpret_cast<const double*>(f32 ? S(0) : K_(0));
     a.fb1 = fc;
-    GT(launch_adj_rho0(h->Kd, a, drho0, G, st));
-    std::vector<double> hp((size_t)(ADJ_NPAR + 2) * G);
+    GT(launch_adj_rho0(h->Kd, a, drho0, Gs, st));
+    std::vector<double> hp((size_t)(ADJ_NPAR + 1) * G + Gs); // pacc, jtne, jmis
     GT(cudaMemcpyAsync(hp.data(), pacc, sizeof(double) * hp.size(), cudaMemcpyDeviceToHost, st));
     if (out->drho0)
         GT(cudaMemcpyAsync(out->drho0, drho0, sizeof(double) * nx, cudaMemcpyDeviceToHost, st));
@@ -1222,7 +1200,8 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
     double sums[ADJ_NPAR + 2];
     for (int q = 0; q < ADJ_NPAR + 2; q++) {
         double s = 0.0;
-        for (int b = 0; b < G; b++) s += hp[(size_t)q * G + b];
+        const int nb = q <= ADJ_NPAR ? G : Gs;
+        for (int b = 0; b < nb; b++) s += hp[(size_t)q * G + b];
         sums[q] = s;
     }
     for (int k = 0; k < 16; k++) out->dS[k] = k < 4 ? 0.0 : sums[k - 4];
