@@ -482,7 +482,7 @@ lbkm_status lbkm_create(const lbkm_params* pin, void* cuda_stream, lbkm_t* out)
             if (e != cudaSuccess) return bail(e, "tensor maps");
         }
     }
-    h->line = line_plan(h->precision, h->nx);
+    h->line = line_plan(h->precision, h->nx, p.tne_every > 0);
     h->grid = h->two_d ? step_grid(h->precision, h->recovery, h->nx, h->ny, sbc, p.tne_every > 0) : h->line.grid;
     if (h->grid < 1) return bail(cudaGetLastError(), "step grid");
     h->tgrid = tne_grid(h->nx, h->ny);
@@ -1119,7 +1119,7 @@ lbkm_status lbkm_grad(lbkm_t h, const lbkm_objective* ob, lbkm_grad_out* out)
     sl.ctr = sctr;
     sl.tne_every = 0;
     LineArgs sd = sl; // the FP64 steps of the recomputed segments: every state is kept
-    const LinePlan dplan = f32 ? line_plan(0, nx) : h->line;
+    const LinePlan dplan = f32 ? line_plan(0, nx, false) : h->line;
     sd.out_stride = (int64_t)(SBd / sizeof(double));
     // forward run in the handle's precision, keeping a state every C steps, up to the last of
     // them: the segment from there is formed below with all its states, the final one included
@@ -1246,7 +1246,7 @@ lbkm_status lbkm_objective_value(lbkm_t h, const lbkm_objective* ob, double* J,
     const size_t nwork = (size_t)nx * (16 + 1 + 1) + (size_t)2 * G;
     // steps per launch: every FP64 state is wanted, so a launch keeps its steps' states in
     // one of two sets of `m`; long grids, whose launches are short of nothing, keep one state
-    const LinePlan dplan = f32 ? line_plan(0, nx) : h->line;
+    const LinePlan dplan = f32 ? line_plan(0, nx, false) : h->line;
     const int m64 = nx <= 65536 ? dplan.steps : 1;
     cudaError_t e = dmalloc(h, &run, f32 ? SBf * 2 : SBd * 2 * m64);
     if (e == cudaSuccess && f32) e = dmalloc(h, &seg, SBd * 2 * m64);

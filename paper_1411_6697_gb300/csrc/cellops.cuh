@@ -135,25 +135,29 @@ __device__ __forceinline__ void deltas(const ModelConst<R>& K, const StepConst<R
     D[6] = fm(-m3, Ta, dot4(K.Bodd + 12, b.ay0, b.ay2, b.ay1, b.ay3));
 }
 
-// W = Omega = M^-1 [-S Delta + A_hat + C_hat] in block form (Omega_hat_1..3 vanish). A8, A9:
-// A_hat_8 and A_hat_9 over rho T; cr: dlambda times the chemical constant, `react`
-// (warp-uniform) if it is nonzero anywhere in the warp.
+// W = Omega = M^-1 [-S Delta + A_hat + C_hat] in block form (Omega_hat_1..3 vanish). S: the
+// rates; A8, A9: A_hat_8 and A_hat_9 over rho T; cr: dlambda times the chemical constant,
+// `react` (warp-uniform) if it is nonzero anywhere in the warp.
 template <typename R>
-__device__ __forceinline__ void collide(const ModelConst<R>& K, const StepConst<R>& E, const R* D, R m1,
+struct Sectors { // M^-1 Omega_hat before the back butterflies
+    R es[4], ea[2], ox[4], oy[4], oo[2];
+};
+template <typename R>
+__device__ __forceinline__ void sectors(const ModelConst<R>& K, const StepConst<R>& E, const R* S, const R* D, R m1,
                                         R m2, R m3, R ux, R uy, R u2, R T, R pT, R A8, R A9, bool react,
-                                        R cr, R* W)
+                                        R cr, Sectors<R>& z)
 {
     R Om[16]; // Omega_hat; the ES and EA sectors already joined (es, ea)
 #pragma unroll
     for (int k = 4; k < 16; k++)
-        if (k != 6 && k != 15) Om[k] = mu(-K.S[k], D[k - 4]);
-    R es2 = fm(-K.S[6], D[2], Om[4]), ea0 = fm(K.S[6], D[2], Om[4]);
-    R es3 = fm(-K.S[15], D[11], Om[13]), ea1 = fm(K.S[15], D[11], Om[13]);
+        if (k != 6 && k != 15) Om[k] = mu(-S[k], D[k - 4]);
+    R es2 = fm(-S[6], D[2], Om[4]), ea0 = fm(S[6], D[2], Om[4]);
+    R es3 = fm(-S[15], D[11], Om[13]), ea1 = fm(S[15], D[11], Om[13]);
     if (E.a_hat) { // Eqs. (3)-(4)
         Om[7] = fm(pT, A8, Om[7]);
         Om[8] = fm(pT, A9, Om[8]);
     }
-    R pes[4], pea[2], px[4], py[4], po[2], e1 = R(0); // e1: Omega_hat_4
+    R *pes = z.es, *pea = z.ea, *px = z.ox, *py = z.oy, *po = z.oo, e1 = R(0); // e1: Omega_hat_4
     if (react) { // C_hat = d f_hat^eq / dT cr (Eqs. (19)-(23))
         const R dA = fm(R(2) * E.di2, T, u2), pd = mu(m1, dA), c4 = E.di2 + R(2);
         const R xx = mu(mu(m2, ux), c4), yy = mu(mu(m3, uy), c4), xy = mu(mu(m2, uy), c4);
@@ -184,6 +188,15 @@ __device__ __forceinline__ void collide(const ModelConst<R>& K, const StepConst<
         pea[r] = fm(K.Iea[2 * r + 1], ea1, mu(K.Iea[2 * r], ea0));
         po[r] = fm(K.Ioo[2 * r + 1], Om[14], mu(K.Ioo[2 * r], Om[5]));
     }
+}
+template <typename R>
+__device__ __forceinline__ void collide(const ModelConst<R>& K, const StepConst<R>& E, const R* S, const R* D, R m1,
+                                        R m2, R m3, R ux, R uy, R u2, R T, R pT, R A8, R A9, bool react,
+                                        R cr, R* W)
+{
+    Sectors<R> z;
+    sectors(K, E, S, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, cr, z);
+    const R *pes = z.es, *pea = z.ea, *px = z.ox, *py = z.oy, *po = z.oo;
 #pragma unroll
     for (int c = 0; c < 2; c++) {
         const R pp = ad(pes[c], pea[c]), pm = ad(pes[c], -pea[c]);

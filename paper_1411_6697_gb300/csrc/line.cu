@@ -17,8 +17,8 @@
 //
 // Measured per step, against one launch per step of a tile kernel with the plain formulas
 // (every stencil's differences, FP64 minmod and FP64 sums of an FP32 state): Sod tube of 400
-// cells FP64 29.8 -> 11.7 us; detonation of 16384 cells FP32 13.3 -> 2.1 us, FP64 with records
-// at every step 58.9 -> 24.9 us.
+// cells FP64 29.8 -> 11.7 us (6.8 with four warps to a window, below); detonation of 16384 cells
+// FP32 13.3 -> 2.1 us, FP64 with records at every step 58.9 -> 24.9 us.
 //
 // Boundaries: lanes past a zero-gradient end are read through the index of the end cell,
 // lanes past a Dirichlet end hold the side's equilibrium, and on a periodic grid every lane
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(LINE_THREADS)
         const bool react = __any_sync(0xffffffffu, hot);
         R dlam = R(0);
         if (react && hot) dlam = reaction_increment(lam, mu(K.omega1, pT), mu(K.omega2, pT), K.dt);
-        collide(K, E, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, mu(dlam, K.chem), W);
+        collide(K, E, K.S, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, mu(dlam, K.chem), W);
         // NND differences (v > 0 from d_{j-2}, d_{j-1}, d_j; v < 0 from d_{j-1}, d_j, d_{j+1};
         // d_j = q_{j+1} - q_j) and the Euler update; lambda's side by the sign of u_x
         if constexpr (sizeof(R) == 8) __syncthreads();
@@ -248,6 +248,190 @@ __global__ void __launch_bounds__(LINE_THREADS)
     }
 }
 
+__device__ __forceinline__ void join_warps() // a barrier that the four warps reach from their own code
+{
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+}
+
+// The FP64 step of a short grid: four warps of one SM share a window of 32 cells, warp r holding
+// the velocities of orbit r and one sector of the moments, so each quarter of the SM runs about
+// 110 FP64 instructions a step instead of 298 while the other three would idle. Butterflies and
+// back-transformed sectors pass through shared memory, two barriers a step; what a cell's
+// neighbours provide stays within the warp (shuffles). The operations and their order are those
+// of line_kernel, so both give the same bits. Bound by that chain of FP64 instructions: Sod tube
+// of 400 cells 11.7 -> 6.8 us per step.
+template <int Q> // the orbit and sector of this warp: 0 ES + EA, 1 OX, 2 OY, 3 OO and lambda
+__device__ __forceinline__ void split_steps(const ModelConst<double>& K, const StepConst<double>& E,
+                                            const LineArgs& a, int kmax, double* bf, double* tr)
+{
+    constexpr bool DIAG = Q & 1;
+    const unsigned all = 0xffffffffu;
+    const int t = threadIdx.x & 31, n = 32, h = 2 * kmax, own = n - 2 * h;
+    const int nx = K.nx, x0 = blockIdx.x * own - h, x = x0 + t;
+    const int64_t plane = K.plane;
+    const double* in = static_cast<const double*>(a.in);
+    int gx = x, dir = -1;
+    bool fixed = false;
+    if (x < 0 || x >= nx) {
+        const int s = x < 0 ? 0 : 1, code = K.sbc[s];
+        if (code == 0) {
+            gx = x % nx;
+            gx = gx < 0 ? gx + nx : gx;
+        } else {
+            gx = x < 0 ? 0 : nx - 1;
+            fixed = true;
+            if (code == 3) dir = s;
+        }
+    }
+    const int lo = K.sbc[0] == 1 && -x0 > 0 ? (-x0 < n ? -x0 : n - 1) : 0;
+    const int hi = K.sbc[1] == 1 && nx - 1 - x0 < n - 1 ? (nx - 1 - x0 > 0 ? nx - 1 - x0 : 0) : n - 1;
+    auto at = [&](int j) { return j < lo ? lo : (j > hi ? hi : j); };
+    const int jm1 = at(t - 1), j0 = at(t), jp1 = at(t + 1);
+    const int dm2 = t >= 2 ? t - 2 : 0, dm1 = t >= 1 ? t - 1 : 0, dp1 = t + 1 < n ? t + 1 : n - 1;
+    const bool mine = t >= h && t < h + own && x < nx;
+
+    double f[4], lam = dir >= 0 ? K.sfeq[dir][16] : in[16 * plane + gx];
+#pragma unroll
+    for (int j = 0; j < 4; j++) f[j] = dir >= 0 ? K.sfeq[dir][4 * Q + j] : in[(4 * Q + j) * plane + gx];
+    int bad = 0;
+    for (int s = 0; s < a.nsteps; s++) {
+        // this orbit's butterflies
+        if constexpr (!DIAG) {
+            const double sx = f[0] + f[2], sy = f[1] + f[3];
+            bf[(4 * Q + 0) * n + t] = sx + sy;
+            bf[(4 * Q + 1) * n + t] = sx - sy;
+            bf[(4 * Q + 2) * n + t] = f[0] - f[2];
+            bf[(4 * Q + 3) * n + t] = f[1] - f[3];
+        } else {
+            const double s01 = f[0] + f[1], d01 = f[0] - f[1], s23 = f[2] + f[3], d23 = f[2] - f[3];
+            bf[(4 * Q + 0) * n + t] = s01 + s23;
+            bf[(4 * Q + 1) * n + t] = d01 + d23;
+            bf[(4 * Q + 2) * n + t] = d01 - d23;
+            bf[(4 * Q + 3) * n + t] = s01 - s23;
+        }
+        if constexpr (Q == 3) bf[16 * n + t] = lam;
+        join_warps();
+        Fly<double> b;
+        {
+            const double* c = bf + t;
+            b.P0 = c[0], b.M0 = c[n], b.ax0 = c[2 * n], b.ay0 = c[3 * n];
+            b.e1 = c[4 * n], b.o1 = c[5 * n], b.ax1 = c[6 * n], b.ay1 = c[7 * n];
+            b.P2 = c[8 * n], b.M2 = c[9 * n], b.ax2 = c[10 * n], b.ay2 = c[11 * n];
+            b.e3 = c[12 * n], b.o3 = c[13 * n], b.ax3 = c[14 * n], b.ay3 = c[15 * n];
+            if constexpr (Q != 3) lam = c[16 * n];
+        }
+        double m1, m2, m3, ux, uy, ux2, uy2, u2, T;
+        bool ok;
+        recover64(K, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, ok);
+        if (mine && !ok) bad = 1;
+        const double pT = mu(m1, T);
+        const bool hot = dbits(T) > dbits(K.T_igd) && dbits(lam) != dbits(1.0);
+        const bool react = __any_sync(all, hot);
+        double dlam = 0.0;
+        if (react && hot) dlam = reaction_increment(lam, mu(K.omega1, pT), mu(K.omega2, pT), K.dt);
+        const double cr = mu(dlam, K.chem);
+        double A8 = 0.0, A9 = 0.0;
+        if ((Q == 1 || Q == 2) && E.a_hat) {
+            const double dux = __shfl_sync(all, ux, jp1) - __shfl_sync(all, ux, jm1);
+            const double duy = __shfl_sync(all, uy, jp1) - __shfl_sync(all, uy, jm1);
+            a_hat<false>(E, ux, uy, dux, duy, 0.0, 0.0, A8, A9);
+        }
+        // this sector's part of the collision (unused entries and rows fall away)
+        double D[TNE_K];
+        deltas(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
+        Sectors<double> z;
+        sectors(K, E, K.S, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, cr, z);
+        if constexpr (Q == 0) {
+#pragma unroll
+            for (int r = 0; r < 4; r++) tr[r * n + t] = z.es[r];
+            tr[4 * n + t] = z.ea[0];
+            tr[5 * n + t] = z.ea[1];
+        } else if constexpr (Q == 3) {
+            tr[14 * n + t] = z.oo[0];
+            tr[15 * n + t] = z.oo[1];
+        } else {
+#pragma unroll
+            for (int r = 0; r < 4; r++) tr[((Q == 1 ? 6 : 10) + r) * n + t] = Q == 1 ? z.ox[r] : z.oy[r];
+        }
+        join_warps();
+        // back to this orbit's velocities, NND differences and the Euler update
+        double W[4];
+        {
+            const double* c = tr + t;
+            constexpr int o = Q >> 1; // axis or diagonal orbit number
+            const double px = c[(6 + (DIAG ? 2 : 0) + o) * n], py = c[(10 + (DIAG ? 2 : 0) + o) * n];
+            if constexpr (!DIAG) {
+                const double es = c[o * n], ea = c[(4 + o) * n];
+                const double pp = ad(es, ea), pm = ad(es, -ea);
+                W[0] = ad(pp, px);
+                W[2] = ad(pp, -px);
+                W[1] = ad(pm, py);
+                W[3] = ad(pm, -py);
+            } else {
+                const double es = c[(2 + o) * n], oo = c[(14 + o) * n];
+                const double eo = ad(es, oo), em = ad(es, -oo), xp = ad(px, py), xm = ad(px, -py);
+                W[0] = ad(eo, xp);
+                W[1] = ad(em, -xm);
+                W[2] = ad(eo, -xp);
+                W[3] = ad(em, xm);
+            }
+        }
+        auto nnd = [&](double q, bool neg) { // d_j = q_{j+1} - q_j, exchanged within the warp
+            const double d = __shfl_sync(all, q, jp1) - __shfl_sync(all, q, j0);
+            const double l2 = __shfl_sync(all, d, dm2), l1 = __shfl_sync(all, d, dm1), r1 = __shfl_sync(all, d, dp1);
+            return neg ? nnd3(l1, d, r1, true) : nnd3(l2, l1, d, false);
+        };
+        double nf[4], nlam = lam;
+#pragma unroll
+        for (int j = 0; j < 4; j++) {
+            const int k = slot_of(4 * Q + j);
+            if (k >= 0) W[j] = fm(k >= 6 ? E.cdx[Q] : -E.cdx[Q], nnd(f[j], k >= 6), W[j]);
+            nf[j] = fm(K.dt, W[j], f[j]);
+        }
+        if constexpr (Q == 3) {
+            const double d = __shfl_sync(all, lam, jp1) - __shfl_sync(all, lam, j0);
+            const double l2 = __shfl_sync(all, d, dm2), l1 = __shfl_sync(all, d, dm1), r1 = __shfl_sync(all, d, dp1);
+            const bool neg = negative(ux);
+            const double X = nnd3(neg ? l1 : l2, neg ? d : l1, neg ? r1 : d, neg);
+            nlam = clamp01(ad(lam, fm(mu(-E.dtdx, ux), X, dlam)));
+        }
+        if (mine && (s == a.nsteps - 1 || a.out_stride > 0)) {
+            double* out = static_cast<double*>(a.out) + (a.out_stride > 0 ? s * a.out_stride : 0) + x;
+            const bool avg = a.stage >= 2;
+            const double* prev = static_cast<const double*>(a.prev) + x;
+            auto put = [&](int i, double v) {
+                out[i * plane] = avg ? fm(a.wprev, prev[i * plane], mu(a.wnew, v)) : v;
+            };
+#pragma unroll
+            for (int j = 0; j < 4; j++) put(4 * Q + j, nf[j]);
+            if constexpr (Q == 3) put(16, nlam);
+        }
+        if (!fixed) {
+#pragma unroll
+            for (int j = 0; j < 4; j++) f[j] = nf[j];
+            lam = nlam;
+        }
+    }
+    if (Q == 0 && __any_sync(all, bad) && t == 0) atomicOr(&a.ctr->status, 1);
+}
+
+__global__ void __launch_bounds__(128)
+    line_split_kernel(const __grid_constant__ ModelConst<double> K, const __grid_constant__ StepConst<double> E,
+                      const __grid_constant__ LineArgs a, int kmax)
+{
+    __shared__ double bf[17 * 32], tr[16 * 32]; // butterflies and lambda; transformed sectors
+    switch (threadIdx.x >> 5) {
+    case 0: split_steps<0>(K, E, a, kmax, bf, tr); break;
+    case 1: split_steps<1>(K, E, a, kmax, bf, tr); break;
+    case 2: split_steps<2>(K, E, a, kmax, bf, tr); break;
+    default: split_steps<3>(K, E, a, kmax, bf, tr); break;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (a.stage < 2) a.ctr->tne_pending = 0;
+        if (a.stage == 0 || a.stage == 2) a.ctr->step += a.nsteps;
+    }
+}
+
 template <typename R, int REC, bool TNE>
 cudaError_t line_launch_t(const ModelConst<R>& K, const LinePlan& p, const LineArgs& a, cudaStream_t s)
 {
@@ -274,7 +458,7 @@ cudaError_t line_launch_t(const ModelConst<R>& K, const LinePlan& p, const LineA
 // 128 threads, one block per SM (FP32 1.80, FP64 14.2; 8 steps, whose 171 blocks no longer
 // fit one per SM, 2.19 and 23.3), and a million cells two FP32 steps (41.5; one 48.3, eight
 // 46.2), one FP64 step (622; four 683).
-LinePlan line_plan(int precision, int nx)
+LinePlan line_plan(int precision, int nx, bool tne)
 {
     static int sms = -1;
     if (sms < 0) {
@@ -282,7 +466,7 @@ LinePlan line_plan(int precision, int nx)
         cudaGetDevice(&dev);
         if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms < 1) sms = 152;
     }
-    LinePlan best = {128, 1, (nx + 123) / 124};
+    LinePlan best = {128, 1, (nx + 123) / 124, false};
     double t_best = 1e300;
     for (int threads = 32; threads <= LINE_THREADS; threads += 32)
         for (int steps = 1; steps <= 16; steps *= 2) {
@@ -292,8 +476,16 @@ LinePlan line_plan(int precision, int nx)
             const double w = (double)((grid + sms - 1) / sms) * (threads / 32);
             const double t = precision == 0 ? (w > 4.25 ? 3.0 * w : 12.8) + 1.5 / steps
                                             : (w > 21.0 ? 0.17 * w : 0.85 + 0.131 * w) + 2.0 / steps;
-            if (t < t_best) t_best = t, best = {threads, steps, grid};
+            if (t < t_best) t_best = t, best = {threads, steps, grid, false};
         }
+    // four warps to a window of 32 cells while every window has an SM of its own (400 cells: 6.8
+    // us per step against 11.7; two windows on an SM would share its FP64 unit and take twice as
+    // long for at most twice the cells of one warp per quarter)
+    for (int steps = 1; precision == 0 && !tne && steps <= 4; steps *= 2) {
+        const int own = 32 - 4 * steps, grid = (nx + own - 1) / own;
+        const double t = 5.0 + 1.5 / steps;
+        if (grid <= sms && t < t_best) t_best = t, best = {128, steps, grid, true};
+    }
     return best;
 }
 
@@ -305,6 +497,13 @@ cudaError_t launch_line(int precision, int recovery, const void* K, const LinePl
     if (a.stage >= 2) b.tne_every = 0; // only u^n has records
     if (precision == 0) {
         const ModelConst<double>& Kd = *static_cast<const ModelConst<double>*>(K);
+        if (p.split) {
+            if (b.tne_every > 0) return cudaErrorInvalidValue;
+            StepConst<double> E;
+            step_const(Kd, &E);
+            line_split_kernel<<<p.grid, 128, 0, s>>>(Kd, E, b, p.steps);
+            return cudaGetLastError();
+        }
         return b.tne_every > 0 ? line_launch_t<double, 0, true>(Kd, p, b, s) : line_launch_t<double, 0, false>(Kd, p, b, s);
     }
     const ModelConst<float>& Kf = *static_cast<const ModelConst<float>*>(K);

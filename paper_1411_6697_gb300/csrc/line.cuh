@@ -11,9 +11,10 @@ namespace lbk {
 // threads - 4 steps are the block's own; `steps` time steps run in one launch.
 struct LinePlan {
     int threads, steps, grid;
+    bool split; // FP64 without records on a short grid: the block's four warps share 32 cells
 };
-// precision: 0 = FP64, 1 = FP32
-LinePlan line_plan(int precision, int nx);
+// precision: 0 = FP64, 1 = FP32; tne: launches may keep records
+LinePlan line_plan(int precision, int nx, bool tne);
 
 struct LineArgs {
     const void* in;        // state at t_n, 17 planes

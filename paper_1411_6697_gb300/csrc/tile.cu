@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(Tile<R>::TT, sizeof(R) == 8 ? 2 : 4)
             const R* v0 = u0 + UH * UW;
             a_hat<true>(E, ux, uy, u0[1] - u0[-1], v0[1] - v0[-1], u0[UW] - u0[-UW], v0[UW] - v0[-UW], A8, A9);
         }
-        collide(K, E, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, mu(dlam, K.chem), W);
+        collide(K, E, K.S, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, mu(dlam, K.chem), W);
 
         // NND flux differences of plane i along one axis (stride d), upwind side by `neg`
         auto nnd = [&](const R* q, R q0, int d, bool neg) -> R {
