@@ -947,6 +947,243 @@ cudaError_t step_launch(const Model<R>& K, const Args& a, int blocks, cudaStream
                       : ((srt) ? CALL(float, true, false, false)                                   \
                          : (tne) ? CALL(float, false, false, true) : CALL(float, false, false, false))))
 
+// ---- short 1-D grids in FP64: four warps to a window of 32 cells -----------------
+// One warp to 32 cells leaves three quarters of each SM's FP64 unit idle on a grid of a few
+// thousand cells. Here warps 0..2 hold the velocities of one speed group each, warp 3 lambda; the moment
+// sectors are shared out as ee (first rows) to warp 0, oe to 1, eo to 2, ee (last rows) and oo to
+// 3. Butterflies, the ee entries and the back-transformed sectors pass through shared memory,
+// three barriers a step; what neighbouring cells provide stays within a warp (shuffles). Up to
+// `kmax` steps run in one launch, of the window all but 2 kmax cells at either end being right
+// after them. The operations and their order are those of step_kernel.
+constexpr int SPLIT_EE = 5; // inverse rows 0..4 of ee in warp 0, Delta rows 2..5; the rest in warp 3
+
+struct SplitShared {
+    double g[NV][32], dx[9][32], dy[9][32], go[NV][32], ge[NV][32], lam[32];
+};
+__device__ __forceinline__ void join_warps() // a barrier that the four warps reach from their own code
+{
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+}
+
+template <int Q>
+__device__ __forceinline__ void split24_steps(const Model<double>& K, const Args& a, int nsteps, int kmax,
+                                              SplitShared& sh)
+{
+    const unsigned all = 0xffffffffu;
+    constexpr int n = 32;
+    const int t = threadIdx.x & 31, h = 2 * kmax, own = n - 2 * h;
+    const int nx = K.nx, x0 = blockIdx.x * own - h, x = x0 + t;
+    const double* in = static_cast<const double*>(a.in);
+    int gx = x, dir = -1;
+    bool fixed = false;
+    if (x < 0 || x >= nx) {
+        const int s = x < 0 ? 0 : 1, code = K.sides[s];
+        if (code == 0) {
+            gx = x % nx;
+            gx = gx < 0 ? gx + nx : gx;
+        } else {
+            gx = x < 0 ? 0 : nx - 1;
+            fixed = true;
+            if (code == 3) dir = s;
+        }
+    }
+    const int lo = K.sides[0] == 1 && -x0 > 0 ? (-x0 < n ? -x0 : n - 1) : 0;
+    const int hi = K.sides[1] == 1 && nx - 1 - x0 < n - 1 ? (nx - 1 - x0 > 0 ? nx - 1 - x0 : 0) : n - 1;
+    auto at = [&](int j) { return j < lo ? lo : (j > hi ? hi : j); };
+    const int jm1 = at(t - 1), j0 = at(t), jp1 = at(t + 1);
+    const int dm2 = t >= 2 ? t - 2 : 0, dm1 = t >= 1 ? t - 1 : 0, dp1 = t + 1 < n ? t + 1 : n - 1;
+    const bool mine = t >= h && t < h + own && x < nx;
+    auto slope3 = [&](double q, double& l2, double& l1, double& d, double& r1) {
+        d = sub(__shfl_sync(all, q, jp1), __shfl_sync(all, q, j0));
+        l2 = __shfl_sync(all, d, dm2);
+        l1 = __shfl_sync(all, d, dm1);
+        r1 = __shfl_sync(all, d, dp1);
+    };
+
+    constexpr int G = Q < 3 ? Q : 0; // the speed group (warp 3: none)
+    double f[8], lam = dir >= 0 ? K.sfeq[dir][NV] : in[(size_t)NV * K.plane + gx];
+    if constexpr (Q < 3) {
+#pragma unroll
+        for (int j = 0; j < 8; j++) f[j] = dir >= 0 ? K.sfeq[dir][8 * G + j] : in[(size_t)(8 * G + j) * K.plane + gx];
+    }
+    int bad = 0;
+    for (int s = 0; s < nsteps; s++) {
+        if constexpr (Q < 3) {
+            const double s02 = f[0] + f[2], s13 = f[1] + f[3];
+            sh.g[3 * G][t] = s02;
+            sh.g[3 * G + 1][t] = s13;
+            sh.g[9 + 2 * G][t] = f[0] - f[2];
+            sh.g[15 + 2 * G][t] = f[1] - f[3];
+            const double ac = f[4] + f[6], bd = f[5] + f[7], am = f[4] - f[6], bm = f[5] - f[7];
+            sh.g[3 * G + 2][t] = ac + bd;
+            sh.g[10 + 2 * G][t] = am - bm;
+            sh.g[16 + 2 * G][t] = am + bm;
+            sh.g[21 + G][t] = ac - bd;
+        } else {
+            sh.lam[t] = lam;
+        }
+        join_warps();
+        double g[NV];
+#pragma unroll
+        for (int p = 0; p < NV; p++) g[p] = sh.g[p][t];
+        if constexpr (Q < 3) lam = sh.lam[t];
+        const Macro m = recover24(K, nullptr, g);
+        if (mine && !m.ok) bad = 1;
+        const Eq24<double> e = eq24(K, m.rho, m.ux, m.uy, m.T);
+        const bool hot = m.hot && dbits(lam) != dbits(1.0);
+        const bool react = __any_sync(all, hot);
+        double dlam = 0.0, chem = 0.0;
+        if (react && hot) {
+            const double pT = mu(m.rho, m.T);
+            dlam = reaction_increment<double>(lam, mu(K.omega1, pT), mu(K.omega2, pT), K.dt);
+            const double rT = lbk::recip64(m.T);
+            chem = mu(mu(K.kchem, dlam), mu(rT, rT));
+        }
+        // this warp's Delta (y) and relaxed entries (w), in sector order
+        double w[NV], y[NV];
+        auto delta = [&](int sct, int r) {
+            const int p = sec_p(sct) + r;
+            y[p] = minus_eq(e, mom_of(p), row_dot(K.Bf, sct, r, 0, g));
+            w[p] = mu(-K.S[mom_of(p)], y[p]);
+        };
+        if constexpr (Q == 0) {
+#pragma unroll
+            for (int r = 2; r < 6; r++) delta(0, r);
+        } else if constexpr (Q == 3) {
+#pragma unroll
+            for (int r = 6; r < 9; r++) delta(0, r);
+#pragma unroll
+            for (int r = 0; r < 3; r++) delta(3, r);
+        } else {
+#pragma unroll
+            for (int r = 1; r < 6; r++) delta(Q, r);
+            const double gxx = mu(sub(__shfl_sync(all, m.ux, jp1), __shfl_sync(all, m.ux, jm1)), K.hdx_r);
+            const double gyx = mu(sub(__shfl_sync(all, m.uy, jp1), __shfl_sync(all, m.uy, jm1)), K.hdx_r);
+            const double th = mu(gxx, K.inv_DI_r), shr = mu(2.0, gyx);
+            if constexpr (Q == 1)
+                w[10] = fm(mu(e.pT, K.A8c_r), fm(m.uy, shr, mu(mu(4.0, m.ux), sub(gxx, th))), w[10]);
+            else
+                w[16] = fm(mu(e.pT, K.A9c_r), fm(m.ux, shr, mu(mu(4.0, m.uy), sub(0.0, th))), w[16]);
+        }
+        if constexpr (Q == 0 || Q == 3) { // the ee entries, wanted by both
+#pragma unroll
+            for (int p = 2; p < 9; p++)
+                if ((p < 6) == (Q == 0)) {
+                    sh.dx[p][t] = w[p];
+                    if (react) sh.dy[p][t] = y[p];
+                }
+        }
+        join_warps();
+        if constexpr (Q == 0 || Q == 3) {
+#pragma unroll
+            for (int p = 2; p < 9; p++)
+                if ((p < 6) != (Q == 0)) {
+                    w[p] = sh.dx[p][t];
+                    if (react) y[p] = sh.dy[p][t];
+                }
+        }
+        auto rows = [&](const double* v, double (*to)[32]) {
+            if constexpr (Q == 0 || Q == 3) {
+#pragma unroll
+                for (int r = 0; r < 9; r++)
+                    if ((r < SPLIT_EE) == (Q == 0)) to[r][t] = row_dot(K.Bis, 0, r, 2, v);
+            }
+            if constexpr (Q == 3) {
+#pragma unroll
+                for (int r = 0; r < 3; r++) to[21 + r][t] = row_dot(K.Bis, 3, r, 0, v);
+            } else if constexpr (Q != 0) {
+#pragma unroll
+                for (int r = 0; r < 6; r++) to[sec_p(Q) + r][t] = row_dot(K.Bis, Q, r, 1, v);
+            }
+        };
+        rows(w, sh.go);
+        if (react) rows(y, sh.ge);
+        join_warps();
+        // back to this group's velocities; chemical term, NND differences, Euler update
+        double nlam = lam;
+        if constexpr (Q < 3) {
+            auto back = [&](const double (*c)[32], double* v) {
+                const double e0 = c[3 * G][t], e1 = c[3 * G + 1][t], ax = c[9 + 2 * G][t], ay = c[15 + 2 * G][t];
+                v[0] = ad(e0, ax);
+                v[1] = ad(e1, ay);
+                v[2] = ad(e0, -ax);
+                v[3] = ad(e1, -ay);
+                const double e2 = c[3 * G + 2][t], o = c[21 + G][t], bx = c[10 + 2 * G][t], by = c[16 + 2 * G][t];
+                const double ep = ad(e2, o), em = ad(e2, -o), xp = ad(bx, by), xm = ad(bx, -by);
+                v[4] = ad(ep, xp);
+                v[5] = ad(em, -xm);
+                v[6] = ad(ep, -xp);
+                v[7] = ad(em, xm);
+            };
+            double W[8];
+            back(sh.go, W);
+            if (react) {
+                double fe[8];
+                back(sh.ge, fe);
+                const double base = fm(K.I_r, e.u2, mu(-3.0, e.IT)), i2 = mu(2.0, K.I_r);
+#pragma unroll
+                for (int o = 0; o < 2; o++) {
+                    const double ao = mu(chem, ad(base, K.chem_o[2 * G + o])), cc = mu(chem, mu(i2, K.c_r[2 * G + o]));
+                    const double bx = mu(cc, m.ux), by = mu(cc, m.uy);
+#pragma unroll
+                    for (int j = 0; j < 4; j++) {
+                        const int i = 8 * G + 4 * o + j, sx = vsign_x(i), sy = vsign_y(i);
+                        double k = ao;
+                        if (sx) k = sx > 0 ? sub(k, bx) : ad(k, bx);
+                        if (sy) k = sy > 0 ? sub(k, by) : ad(k, by);
+                        W[4 * o + j] = fm(sub(f[4 * o + j], fe[4 * o + j]), k, W[4 * o + j]);
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; j++) {
+                const int i = 8 * G + j;
+                if (vsign_x(i)) {
+                    double l2, l1, d, r1;
+                    slope3(f[j], l2, l1, d, r1);
+                    const double X = vsign_x(i) < 0 ? lbk::nnd3(l1, d, r1, true) : lbk::nnd3(l2, l1, d, false);
+                    W[j] = fm(-K.vxs[i], X, W[j]);
+                }
+                W[j] = fm(K.dt_r, W[j], f[j]);
+                if (!fixed) f[j] = W[j];
+            }
+        } else {
+            double l2, l1, d, r1;
+            slope3(lam, l2, l1, d, r1);
+            const bool neg = lbk::negative(m.ux);
+            const double X = lbk::nnd3(neg ? l1 : l2, neg ? d : l1, neg ? r1 : d, neg);
+            nlam = lbk::clamp01(ad(lam, fm(mu(mu(-K.dt_r, K.inv_dx_r), m.ux), X, dlam)));
+            if (!fixed) lam = nlam;
+        }
+    }
+    if (mine) {
+        double* out = static_cast<double*>(a.out) + x;
+        if constexpr (Q < 3) {
+#pragma unroll
+            for (int j = 0; j < 8; j++) out[(size_t)(8 * G + j) * K.plane] = f[j];
+        } else {
+            out[(size_t)NV * K.plane] = lam;
+        }
+    }
+    if (Q == 3 && __any_sync(all, bad) && t == 0) atomicOr(&a.ctr->status, 1);
+}
+
+__global__ void __launch_bounds__(128)
+    split_kernel(const __grid_constant__ Model<double> K, const __grid_constant__ Args a, int nsteps, int kmax)
+{
+    __shared__ SplitShared sh;
+    switch (threadIdx.x >> 5) {
+    case 0: split24_steps<0>(K, a, nsteps, kmax, sh); break;
+    case 1: split24_steps<1>(K, a, nsteps, kmax, sh); break;
+    case 2: split24_steps<2>(K, a, nsteps, kmax, sh); break;
+    default: split24_steps<3>(K, a, nsteps, kmax, sh); break;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.ctr->tne_pending = 0;
+        a.ctr->step += nsteps;
+    }
+}
+
 // TNE of a state on demand: Delta fields (optional) and block partials.
 template <typename R>
 __global__ void __launch_bounds__(BT) tne_kernel(const Model<R> K, const R* __restrict__ in,
@@ -1320,6 +1557,7 @@ struct lbkm24 {
     int nblocks;       // of tne_kernel
     dim3 grid, block;
     int sblocks;       // of a step
+    int split;         // > 0: steps per launch of split_kernel (short FP64 1-D grids)
     DevCounters* ctr;
     Record* hist;
     Record* tne_out;
@@ -1353,7 +1591,9 @@ lbkm_status fail(lbkm24_t h, lbkm_status st, const char* fmt, ...)
                         "%s: %s (%s:%d)", #call, cudaGetErrorString(e_), __FILE__, __LINE__); \
     } while (0)
 
-cudaError_t launch_one_step(const lbkm24* h, int from, cudaStream_t st)
+// one step from buf[from], or up to h->split steps in one launch of split_kernel: n comes in as
+// the steps wanted and goes out as the steps launched
+cudaError_t launch_steps(const lbkm24* h, int from, int64_t& n, cudaStream_t st)
 {
     Args a;
     a.in = h->buf[from];
@@ -1364,6 +1604,13 @@ cudaError_t launch_one_step(const lbkm24* h, int from, cudaStream_t st)
     a.hist_cap = h->p.tne_capacity;
     a.tne_every = h->p.tne_every;
     a.area = h->p.dx * h->p.dy;
+    if (h->split) {
+        if (n > h->split) n = h->split;
+        const int own = 32 - 4 * h->split;
+        split_kernel<<<(h->p.nx + own - 1) / own, 128, 0, st>>>(h->Kd, a, (int)n, h->split);
+        return cudaGetLastError();
+    }
+    n = 1;
     if (h->has_wall) {
         const int g = (2 * h->p.nx + 127) / 128;
         if (h->p.precision == LBKM_F64)
@@ -1384,6 +1631,19 @@ cudaError_t launch_one_step(const lbkm24* h, int from, cudaStream_t st)
         e = cudaGetLastError();
     }
     return e;
+}
+
+// Steps per launch of split_kernel, or 0 where it does not apply: FP64, 1-D, moment form, no
+// records, and at most three windows an SM (a window's four warps use all of an SM's FP64 unit,
+// step_kernel's one warp a quarter). 5000 cells, two windows on some SMs: 37.1 us per step with
+// step_kernel, 21.6 with this.
+int split_steps_for(const lbkm24* h, int sms)
+{
+    if (h->p.precision != LBKM_F64 || h->p.ny != 1 || h->srt || h->p.tne_every > 0) return 0;
+    const int nx = h->p.nx;
+    for (int k = 4; k >= 1; k /= 2)
+        if ((nx + 31 - 4 * k) / (32 - 4 * k) <= sms) return k;
+    return (nx + 27) / 28 <= 3 * sms ? 1 : 0;
 }
 
 // streaming multiprocessors of the current device (152 on GB300, the value taken if the
@@ -1580,6 +1840,7 @@ lbkm_status lbkm24_create(const lbkm24_params* pin, void* cuda_stream, lbkm24_t*
     h->sblocks = V24_VARIANT(V24_BLOCKS, p.precision == LBKM_F64, h->srt, p.ny > 1, p.tne_every > 0);
 #undef V24_BLOCKS
     if (h->sblocks < 1) return bail(cudaGetLastError(), "step kernel");
+    h->split = split_steps_for(h, sms);
     const size_t sb = (size_t)NP * h->plane_elems * h->elem;
     for (int k = 0; k < 2; k++)
         if ((ce = cudaMalloc(&h->buf[k], sb)) != cudaSuccess) return bail(ce, "state");
@@ -1674,8 +1935,11 @@ lbkm_status lbkm24_step(lbkm24_t h, int64_t n)
             cudaGraph_t gr;
             TRY24(h, cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal));
             cudaError_t le = cudaSuccess;
-            for (int s = 0; s < GRAPH_CHUNK && le == cudaSuccess; s++)
-                le = launch_one_step(h, (h->cur + s) & 1, h->capture_stream);
+            int c = h->cur;
+            for (int64_t left = GRAPH_CHUNK, m; left > 0 && le == cudaSuccess; left -= m, c = 1 - c) {
+                m = left;
+                le = launch_steps(h, c, m, h->capture_stream);
+            }
             cudaError_t ce = cudaStreamEndCapture(h->capture_stream, &gr);
             if (le != cudaSuccess || ce != cudaSuccess) {
                 if (ce == cudaSuccess) cudaGraphDestroy(gr);
@@ -1691,10 +1955,12 @@ lbkm_status lbkm24_step(lbkm24_t h, int64_t n)
         n -= GRAPH_CHUNK;
         h->host_steps += GRAPH_CHUNK;
     }
-    for (; n > 0; n--) {
-        TRY24(h, launch_one_step(h, h->cur, h->stream));
+    while (n > 0) {
+        int64_t m = n;
+        TRY24(h, launch_steps(h, h->cur, m, h->stream));
         h->cur = 1 - h->cur;
-        h->host_steps++;
+        h->host_steps += m;
+        n -= m;
     }
     return LBKM_OK;
 }

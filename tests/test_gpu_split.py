@@ -6,6 +6,9 @@ import numpy as np
 import pytest
 
 from paper_1411_6697_gb300 import lbkm
+from test_gpu_d2v24 import SIDES
+from test_gpu_d2v24 import mixed_2d as mixed24
+from test_gpu_d2v24 import start as start24
 from test_gpu_line import ENDS
 from test_gpu_parity import mixed_2d, start
 
@@ -25,3 +28,18 @@ def test_line_split_same_bits(nx, ends):
         b.step(n)
     assert np.array_equal(a.f_planes(), b.f_planes())
     assert a.steps_taken == b.steps_taken == 41
+
+
+@pytest.mark.parametrize("bc", [0, 1, 5])
+@pytest.mark.parametrize("nx", [3, 28, 29, 2432, 2433, 3648, 3649, 12768, 12769])
+def test_d2v24_split_same_bits(nx, bc):
+    cfg = mixed24(nx, 1, bc=(bc, 0), seed=nx)
+    if bc == 5:
+        for key in ("params", "lib_params"):
+            cfg[key]["sides"] = SIDES[:2] + [SIDES[1]] * 2
+    a, _, _, _ = start24(cfg, lbkm.F64, noise_seed=5)
+    b, _, _, _ = start24(cfg, lbkm.F64, noise_seed=5, tne_every=64, tne_capacity=4)
+    for n in (37, 1, 3):
+        a.step(n)
+        b.step(n)
+    assert np.array_equal(a.f_planes(), b.f_planes())
