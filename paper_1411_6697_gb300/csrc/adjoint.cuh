@@ -4,6 +4,22 @@
 
 namespace lbk {
 
+constexpr int ADJ_NPAR = 15; // dJ/dS_5..S_16, dJ/dQ, dJ/domega1, dJ/domega2
+struct AdjArgs {
+    const double* f;     // a state: 17 planes with the handle's pitch
+    const double* fb1;   // dJ/df of it, [16][nx] (launch_adj_rho0)
+    double *fb0, *lb0;   // dJ/df and dJ/dlambda of the final state (launch_adj_seed)
+    double* jacc;        // [grid] per-block objective accumulators
+    double jw;           // w_tne dx dt for the objective value
+};
+int adj_grid(int nx);
+cudaError_t launch_adj_seed(const ModelConst<double>& K, const AdjArgs& a, const double* rho_t,
+                            double w, int grid, cudaStream_t s);
+cudaError_t launch_adj_rho0(const ModelConst<double>& K, const AdjArgs& a, double* drho0,
+                            int grid, cudaStream_t s);
+// n floats widened to doubles (an FP32 forward run's checkpoint, to restart a segment in FP64)
+cudaError_t launch_adj_widen(const float* in, double* out, size_t n, int grid, cudaStream_t s);
+
 // How the reverse sweep cuts a grid: blocks of `threads` cells, of which the middle
 // threads - 4 steps - 4 are the block's own, `steps` reverse steps per launch.
 struct AdjPlan {

@@ -791,6 +791,11 @@ lbkm_status lbkm_get_state(lbkm_t h, void* dst, int on_device)
     if (!h || !dst) return LBKM_EINVAL;
     if (!h->initialized) return fail(h, LBKM_ESTATE, "lbkm_get_state before lbkm_init_fields");
     const size_t row = (size_t)h->nx * h->elem, plane = row * h->ny;
+    if (on_device && can_pack((int)h->elem, dst)) {
+        CUDA_TRY(h, launch_pack((int)h->elem, NPLANE, h->buf[h->cur], (int64_t)h->plane_elems, h->pitch, h->nx,
+                                h->ny, dst, h->host_steps, h->stream));
+        return check_status(h);
+    }
     cudaMemcpyKind k = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     for (int pl = 0; pl < NPLANE; pl++)
         CUDA_TRY(h, cudaMemcpy2DAsync((char*)dst + pl * plane, row,

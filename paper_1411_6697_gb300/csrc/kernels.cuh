@@ -73,6 +73,11 @@ cudaError_t launch_init(int precision, const ModelConst<double>& Kd, const doubl
 cudaError_t launch_macros(int precision, const ModelConst<double>& Kd, const void* state,
                           double* rho, double* ux, double* uy, double* T, double* p,
                           double* lam, cudaStream_t s);
+// A state snapshot on the device: `planes` planes of ny rows of nx elements (4 or 8 bytes) packed
+// into dst, then the step counter; for the destinations that can_pack accepts.
+bool can_pack(int elem, const void* dst);
+cudaError_t launch_pack(int elem, int planes, const void* state, int64_t plane_elems, int pitch, int nx,
+                        int ny, void* dst, int64_t step, cudaStream_t s);
 // TNE fields (optional) and grid-wide record of a state, all FP64.
 cudaError_t launch_tne(int precision, const ModelConst<double>& Kd, const void* state,
                        double* delta, double* partials, int grid, DevCounters* ctr,
@@ -110,36 +115,6 @@ cudaError_t launch_batch(int recovery, int block_threads, const ModelConst<float
 cudaError_t launch_tne_instances(int precision, const ModelConst<double>& Kd, const void* state,
                                  const InstParam* inst, int n_inst, TneRecord* out,
                                  double area, cudaStream_t s);
-
-// Discrete adjoint of the FP64 1-D step (adjoint.cu).
-constexpr int ADJ_NPAR = 15; // dJ/dS_5..S_16, dJ/dQ, dJ/domega1, dJ/domega2
-struct AdjArgs {
-    const double* f;     // state n: 17 planes with the handle's pitch
-    const double* mac;   // [4][nx] rho, ux, uy, T of state n
-    const double* fb1;   // dJ/df of state n+1, [16][nx]
-    const double* lb1;   // dJ/dlambda of state n+1, [nx]
-    double* mb;          // [16][nx] pass A -> B: adjoint of the moments
-    double* loc;         // [6][nx] pass A -> B: rho_b, ux_b, uy_b, T_b, lambda_b, clamped lambda_b
-    double* gb;          // [2][nx] pass A -> B: adjoints of du_x/dx, du_y/dx
-    double* cw;          // [17][5][nx] pass A -> B: weighted NND coefficients of each cell's
-                         // stencil (planes f_1..f_16, lambda; offsets -2..+2)
-    double* fb0;         // dJ/df of state n, [16][nx]
-    double* lb0;         // dJ/dlambda of state n, [nx]
-    double* pacc;        // [ADJ_NPAR][grid] per-block parameter accumulators
-    double* jacc;        // [grid] per-block objective accumulators
-    const double* vx;    // [16] x-velocities (M, M^-1 and their transposes act in block form)
-    double tne_w;        // w_tne dx dt: Delta_b += 2 tne_w Delta
-    double jw;           // w_tne dx dt for the objective value
-};
-int adj_grid(int nx);
-cudaError_t launch_adj_step(const ModelConst<double>& K, const AdjArgs& a, int grid,
-                            cudaStream_t s);
-cudaError_t launch_adj_seed(const ModelConst<double>& K, const AdjArgs& a, const double* rho_t,
-                            double w, int grid, cudaStream_t s);
-cudaError_t launch_adj_rho0(const ModelConst<double>& K, const AdjArgs& a, double* drho0,
-                            int grid, cudaStream_t s);
-// n floats widened to doubles (an FP32 forward run's checkpoint, to restart a segment in FP64)
-cudaError_t launch_adj_widen(const float* in, double* out, size_t n, int grid, cudaStream_t s);
 
 // FP32 2-D step: y-marching strips, two cells per thread (march.cu)
 // mode = recovery | (general side conditions << 1) | (single relaxation time << 2) | (TNE << 3)
