@@ -638,7 +638,7 @@ lbkm_status lbkm_step(lbkm_t h, int64_t n)
             CUDA_TRY(h, cudaMemsetAsync(h->d_bar, 0, 2 * sizeof(unsigned), h->stream));
             CUDA_TRY(h, launch_batch(h->recovery, h->bt, h->Kf, batch_args(h, (int)n), h->bgrid,
                                      h->stream));
-            h->cur ^= (int)(n & 1);
+            h->cur ^= batch_phases((int)n) & 1;
             h->host_steps += n;
         }
         return LBKM_OK;

@@ -1,37 +1,52 @@
 // batch.cu -- persistent driver for many 1-D instances of uneven length.
 //
-// The instances are concatenated into one flat grid (each starts on a 16-byte
-// boundary: nx is a multiple of 4). Work items are (instance, segment of 2*BT
-// cells). One launch runs `nsteps` time steps: in each step the blocks walk the
-// item list (grid-stride), staging segment + halo of the 17 planes with
-// double-buffered cp.async copies, recovering rho, u, T of the segment and its
-// two neighbours, and updating two cells per thread with packed FP32 pairs;
-// boundaries are zero-gradient per instance, S, Q and omega1 per instance. A
-// grid barrier separates the steps; its wait is bounded in time and reports a
-// timeout through the status word instead of hanging. The launch is
-// cooperative, so all blocks are resident.
+// The instances are concatenated into one flat grid (each starts on a 16-byte boundary: nx is a
+// multiple of 4). Work items are (instance, segment). One launch runs `nsteps` time steps in
+// phases of up to BATCH_STEPS: in a phase the blocks walk the item list (grid-stride), and a
+// block carries a window of BT cells of its item, one per thread, through the phase's steps in
+// registers, neighbours meeting in shared memory once per step; the middle BT - 4 BATCH_STEPS
+// cells are the item's segment, the rest overlaps with the neighbour items' windows. Boundaries
+// are zero-gradient per instance, S, Q and omega1 per instance. A grid barrier separates the
+// phases; its wait is bounded in time and reports a timeout through the status word instead of
+// hanging. The launch is cooperative, so all blocks are resident.
+//
+// What bounds it: instruction issue and the FP64 unit of the recovery (13 of its instructions a
+// warp and step, 64 cycles each). Two steps per pass took half the state's traffic and half the
+// barriers off; one cell per thread instead of a pair leaves registers for six blocks of 128 on
+// an SM. 512 detonations, 7.95 M cells, ms per step: one step per pass and a pair of cells per
+// thread 0.430; one cell and two steps 0.330 (four 0.361: the shared edges grow; five or eight
+// blocks an SM 0.356, 0.333).
 #include <float.h>
 #include <stdint.h>
 
-#include "cell.cuh"
+#include "cellops.cuh"
 #include "kernels.cuh"
-#include "pair.cuh"
-#include "vec2.cuh"
 
 namespace lbk {
 
 namespace {
 
+constexpr int BATCH_STEPS = 2; // time steps between grid barriers
+constexpr int BNX = 13;        // planes that neighbours read: those with v_x != 0, and lambda
+
+// plane of a slot (v_x > 0 in the first six, v_x < 0 in the next six, then lambda) and the slot
+// of a plane (-1: v_x = 0)
+__host__ __device__ constexpr int slot_plane(int s)
+{
+    constexpr int t[BNX] = {0, 4, 7, 8, 12, 15, 2, 5, 6, 10, 13, 14, 16};
+    return t[s];
+}
+__host__ __device__ constexpr int slot_of(int plane)
+{
+    constexpr int t[16] = {0, -1, 6, -1, 1, 7, 8, 2, 3, -1, 9, -1, 4, 10, 11, 5};
+    return t[plane];
+}
+
 template <int BT>
 struct BCfg {
-    static constexpr int SEG = 2 * BT;           // cells per item
-    static constexpr int SW = SEG + 8;           // staged: x0-4 .. x0+SEG+3
-    static constexpr int CH = SW / 4;            // 16-byte chunks per plane
-    static constexpr int MWB = SEG + 4;          // macro row: x0-2 .. x0+SEG+1
-    static constexpr size_t OFF_MAC = (size_t)2 * NPLANE * SW * 4;
-    static constexpr size_t OFF_IGN = OFF_MAC + (size_t)4 * MWB * 4;
-    static constexpr size_t OFF_PAR = (OFF_IGN + SEG + 15) / 16 * 16;
-    static constexpr size_t SMEM = OFF_PAR + 32 * 4;
+    static constexpr int H = 2 * BATCH_STEPS, SEG = BT - 2 * H; // halo and own cells of an item
+    static constexpr int PUB = (BNX + 2) * BT;                  // published planes, u_x, u_y
+    static constexpr size_t SMEM = sizeof(float) * (2 * PUB + 32);
 };
 
 __device__ __forceinline__ uint64_t global_ns()
@@ -74,195 +89,96 @@ __device__ bool grid_barrier(const BatchLaunch& b, unsigned expected)
     return ok != 0;
 }
 
-template <int BT>
-__device__ __forceinline__ void stage_item(const float* __restrict__ in, float* buf,
-                                           const InstParam& ip, int x0, int64_t plane)
-{
-    using C = BCfg<BT>;
-    for (int c = threadIdx.x; c < NPLANE * C::CH; c += BT) {
-        const int p = c / C::CH, ch = c - p * C::CH;
-        const int x = x0 - 4 + 4 * ch;
-        float* dst = buf + p * C::SW + 4 * ch;
-        const float* src = in + p * plane + ip.off;
-        if (x >= 0 && x + 4 <= ip.nx) {
-            cp16(dst, src + x);
-        } else {
-#pragma unroll
-            for (int e = 0; e < 4; e++) {
-                int xe = x + e;
-                xe = xe < 0 ? 0 : (xe >= ip.nx ? ip.nx - 1 : xe);
-                dst[e] = src[xe];
-            }
-        }
-    }
-}
-
 template <int REC, int BT>
-__global__ void __launch_bounds__(BT)
-    batch_kernel(const ModelConst<float> K, const BatchLaunch b)
+__global__ void __launch_bounds__(BT, 768 / BT)
+    batch_kernel(const __grid_constant__ ModelConst<float> K, const __grid_constant__ StepConst<float> E,
+                 const __grid_constant__ BatchLaunch b)
 {
     using C = BCfg<BT>;
-    extern __shared__ __align__(16) unsigned char smem[];
-    float* stage = reinterpret_cast<float*>(smem);
-    float* mac = reinterpret_cast<float*>(smem + C::OFF_MAC); // rho, ux, uy, T [4][MWB]
-    unsigned char* ign = smem + C::OFF_IGN;
-    float* par = reinterpret_cast<float*>(smem + C::OFF_PAR); // S[16], A8c, A9c, chem, om1, om2
-    const int tid = threadIdx.x;
-    const int lx = 2 * tid + 4, mi = 2 * tid + 2;
-    const DfConst Cd = df_constants(K);
-    const float dt = K.dt;
+    extern __shared__ __align__(16) float sm[];
+    float* par = sm + 2 * C::PUB; // S[16], A8c, A9c, chem, om1, om2
+    const int t = threadIdx.x;
     const unsigned expected = gridDim.x + (unsigned)b.phantom_blocks;
-    int bad = 0;
+    const int64_t plane = K.plane;
 
-    for (int s = 0; s < b.nsteps; s++) {
-        const float* __restrict__ in = static_cast<const float*>(b.buf[(b.cur + s) & 1]);
-        float* __restrict__ out = static_cast<float*>(b.buf[(b.cur + s + 1) & 1]);
-        int cb = 0;
-        int item = blockIdx.x;
-        if (item < b.nitems) {
-            const BatchItem it = b.items[item];
-            stage_item<BT>(in, stage, b.inst[it.inst], it.x0, K.plane);
-        }
-        cp_commit();
-        for (; item < b.nitems; item += gridDim.x) {
-            const int nxt = item + gridDim.x;
-            if (nxt < b.nitems) {
-                const BatchItem it2 = b.items[nxt];
-                stage_item<BT>(in, stage + (cb ^ 1) * NPLANE * C::SW, b.inst[it2.inst], it2.x0,
-                               K.plane);
-            }
-            cp_commit();
+    int phase = 0;
+    for (int done = 0; done < b.nsteps; phase++) {
+        const int m = b.nsteps - done < BATCH_STEPS ? b.nsteps - done : BATCH_STEPS;
+        const bool odd = (b.cur + phase) & 1;
+        const float* __restrict__ in = static_cast<const float*>(odd ? b.buf[1] : b.buf[0]);
+        float* __restrict__ out = static_cast<float*>(odd ? b.buf[0] : b.buf[1]);
+        int bad = 0;
+        for (int item = blockIdx.x; item < b.nitems; item += gridDim.x) {
             const BatchItem it = b.items[item];
             const InstParam& ip = b.inst[it.inst];
-            if (tid < 16) par[tid] = ip.S[tid];
-            if (tid == 16) par[16] = ip.A8c;
-            if (tid == 17) par[17] = ip.A9c;
-            if (tid == 18) par[18] = ip.chem;
-            if (tid == 19) par[19] = ip.om1;
-            if (tid == 20) par[20] = ip.om2;
-            cp_wait<1>();
-            __syncthreads();
-            const float* sb = stage + cb * NPLANE * C::SW;
-            const int cx = it.x0 + 2 * tid;
-            const bool act0 = cx < ip.nx, act1 = cx + 1 < ip.nx;
-
-            // rho, u, T of the two cells (conserved moments, Eqs. (5)-(7)) and halo u
-            {
-                V2 f[16];
+            const int w0 = it.x0 - C::H, x = w0 + t, nx = ip.nx;
+            const int gx = x < 0 ? 0 : (x >= nx ? nx - 1 : x);
+            const bool fixed = x != gx; // a ghost lane: read through the end cell, never updated
+            const bool mine = t >= C::H && t < C::H + C::SEG && x < nx;
+            const int lo = w0 < 0 ? -w0 : 0, hi = nx - 1 - w0 < BT - 1 ? nx - 1 - w0 : BT - 1;
+            auto at = [&](int j) { return j < lo ? lo : (j > hi ? hi : j); };
+            const int jm2 = at(t - 2), jm1 = at(t - 1), jp1 = at(t + 1), jp2 = at(t + 2);
+            const float* src = in + ip.off + gx;
+            float f[16], lam = src[16 * plane];
 #pragma unroll
-                for (int i = 0; i < 16; i++) f[i] = ldv(sb + i * C::SW + lx);
-                V2 rho, ux, uy, T;
-                bool ig0, ig1, ok0, ok1;
-                recover_pair_fast<REC>(f, Cd, K, rho, ux, uy, T, ig0, ig1, ok0, ok1);
-                if ((act0 && !ok0) || (act1 && !ok1)) bad = 1;
-                *reinterpret_cast<float2*>(mac + 0 * C::MWB + mi) = rho.v;
-                *reinterpret_cast<float2*>(mac + 1 * C::MWB + mi) = ux.v;
-                *reinterpret_cast<float2*>(mac + 2 * C::MWB + mi) = uy.v;
-                *reinterpret_cast<float2*>(mac + 3 * C::MWB + mi) = T.v;
-                ign[2 * tid] = ig0;
-                ign[2 * tid + 1] = ig1;
-                if (tid == 0 || tid == BT - 1) {
-                    const int hx = tid == 0 ? 3 : C::SEG + 4;
-                    const int hm = tid == 0 ? 1 : C::SEG + 2;
-                    float g[16];
+            for (int i = 0; i < 16; i++) f[i] = src[i * plane];
+            __syncthreads(); // the previous item is done with shared memory
+            if (t < 16) par[t] = ip.S[t];
+            if (t == 16) par[16] = ip.A8c;
+            if (t == 17) par[17] = ip.A9c;
+            if (t == 18) par[18] = ip.chem;
+            if (t == 19) par[19] = ip.om1;
+            if (t == 20) par[20] = ip.om2;
+            for (int s = 0; s < m; s++) {
+                float* P = sm + (s & 1) * C::PUB;
+                const Fly<float> fl = butterflies(f);
+                float m1, ux, uy, T;
+                bool hot, ok;
+                recover32<REC>(K, f, m1, ux, uy, T, hot, ok);
+                if (mine && !ok) bad = 1;
+                hot = hot && lam != 1.f;
+                const float m2 = mu(m1, ux), m3 = mu(m1, uy);
+                const float ux2 = mu(ux, ux), uy2 = mu(uy, uy), u2 = ad(ux2, uy2), pT = mu(m1, T);
 #pragma unroll
-                    for (int i = 0; i < 16; i++) g[i] = sb[i * C::SW + hx];
-                    float hu, hv;
-                    velocity_f32(g, K, hu, hv);
-                    mac[1 * C::MWB + hm] = hu;
-                    mac[2 * C::MWB + hm] = hv;
-                }
-            }
-            __syncthreads();
-
-            // update of the two cells
-            {
-                V2 f[16];
-#pragma unroll
-                for (int i = 0; i < 16; i++) f[i] = ldv(sb + i * C::SW + lx);
-                const V2 lam0 = ldv(sb + 16 * C::SW + lx);
-                const V2 rho = ldv(mac + 0 * C::MWB + mi), ux = ldv(mac + 1 * C::MWB + mi);
-                const V2 uy = ldv(mac + 2 * C::MWB + mi), T = ldv(mac + 3 * C::MWB + mi);
-                V2 m[16], q[16], D[TNE_K];
-                forward_moments(K, f, m);
-                feq_moments(V2(K.DI), rho, ux, uy, T, q);
-#pragma unroll
-                for (int k = 0; k < TNE_K; k++) D[k] = m[k + 4] - q[k + 4];
-                const float2 uxl = *reinterpret_cast<const float2*>(mac + 1 * C::MWB + mi - 2);
-                const float2 uxh = *reinterpret_cast<const float2*>(mac + 1 * C::MWB + mi + 2);
-                const float2 uyl = *reinterpret_cast<const float2*>(mac + 2 * C::MWB + mi - 2);
-                const float2 uyh = *reinterpret_cast<const float2*>(mac + 2 * C::MWB + mi + 2);
-                const V2 dux_dx = (V2(ux.y(), uxh.x) - V2(uxl.y, ux.x())) * K.half_inv_dx;
-                const V2 duy_dx = (V2(uy.y(), uyh.x) - V2(uyl.y, uy.x())) * K.half_inv_dx;
-                const V2 theta = dux_dx * K.inv_DI;
-                const V2 rT = rho * T;
-                const V2 A8 = (rT * par[16]) * fma(V2(4.f) * ux, dux_dx - theta, V2(2.f) * uy * duy_dx);
-                const V2 A9 = (rT * par[17]) * fma(V2(4.f) * uy, -theta, V2(2.f) * ux * duy_dx);
-                // both cells evaluated, then selected: no divergent branch
-                const float ri0 = reaction_increment(lam0.x(), par[19] * rT.x(), par[20] * rT.x(), dt);
-                const float ri1 = reaction_increment(lam0.y(), par[19] * rT.y(), par[20] * rT.y(), dt);
-                const float dl0 = ign[2 * tid] ? ri0 : 0.f, dl1 = ign[2 * tid + 1] ? ri1 : 0.f;
-                const V2 dlam(dl0, dl1);
-                const V2 cr = dlam * par[18];
-                V2 dq[16], Om[16], W[16];
-                dfeq_dT(V2(K.DI), rho, ux, uy, T, dq);
-                Om[0] = Om[1] = Om[2] = V2(0.f);
-                Om[3] = dq[3] * cr;
-#pragma unroll
-                for (int k = 4; k < 16; k++) Om[k] = fma(V2(-par[k]), D[k - 4], dq[k] * cr);
-                Om[7] += A8;
-                Om[8] += A9;
-                inverse_moments(K, Om, W);
-
-                const Q6 lq = load6(sb + 16 * C::SW, lx);
-                const V2 lpx = nnd_pos_x(lq), lnx = nnd_neg_x(lq);
-                const V2 lax(ux.x() > 0.f ? lpx.x() : lnx.x(), ux.y() > 0.f ? lpx.y() : lnx.y());
-                V2 ln = fma(V2(-dt), ux * K.inv_dx * lax, lam0) + dlam;
-                ln = vmin(vmax(ln, V2(0.f)), V2(1.f));
-
-                const int64_t g = ip.off + cx;
-                auto put = [&](int i, V2 adv) {
-                    const V2 v = fma(V2(dt), W[i] - adv, f[i]);
-                    if (act1)
-                        *reinterpret_cast<float2*>(out + i * K.plane + g) = v.v;
-                    else if (act0)
-                        out[i * K.plane + g] = v.x();
+                for (int k = 0; k < BNX; k++) P[k * BT + t] = slot_plane(k) == 16 ? lam : f[slot_plane(k) & 15];
+                P[BNX * BT + t] = ux;
+                P[(BNX + 1) * BT + t] = uy;
+                __syncthreads();
+                float D[TNE_K], W[16], A8, A9;
+                deltas(K, E, fl, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
+                a_hat<false>(E, ux, uy, P[BNX * BT + jp1] - P[BNX * BT + jm1],
+                             P[(BNX + 1) * BT + jp1] - P[(BNX + 1) * BT + jm1], 0.f, 0.f, A8, A9);
+                const bool react = __any_sync(0xffffffffu, hot);
+                float dlam = 0.f;
+                if (react && hot) dlam = reaction_increment(lam, mu(par[19], pT), mu(par[20], pT), K.dt);
+                collide(K, E, par, D, m1, m2, m3, ux, uy, u2, T, pT, mu(par[16], A8), mu(par[17], A9), react,
+                        mu(dlam, par[18]), W);
+                auto nnd = [&](int k, float q, bool neg) -> float {
+                    const float* r = P + k * BT;
+                    const float l = r[jm1], g = r[jp1];
+                    return neg ? nnd3(q - l, g - q, r[jp2] - g, true) : nnd3(l - r[jm2], q - l, g - q, false);
                 };
-#define PX(i) nnd_pos_x(load6(sb + (i) * C::SW, lx))
-#define NX(i) nnd_neg_x(load6(sb + (i) * C::SW, lx))
 #pragma unroll
-                for (int o = 0; o < 2; o++) { // axis orbits: only (+-c, 0) move along x
-                    const int i0 = 8 * o;
-                    const float cxs = K.c[2 * o] * K.inv_dx;
-                    put(i0 + 0, cxs * PX(i0 + 0));
-                    put(i0 + 1, V2(0.f));
-                    put(i0 + 2, -cxs * NX(i0 + 2));
-                    put(i0 + 3, V2(0.f));
+                for (int i = 0; i < 16; i++) { // the increment first: one rounding at the size of f
+                    const int k = slot_of(i);
+                    float w = mu(K.dt, W[i]);
+                    if (k >= 0) w = fm(k >= 6 ? E.cdx[i >> 2] : -E.cdx[i >> 2], nnd(k, f[i], k >= 6), w);
+                    if (!fixed) f[i] = ad(f[i], w);
                 }
-#pragma unroll
-                for (int o = 0; o < 2; o++) { // diagonal orbits
-                    const int i0 = 4 + 8 * o;
-                    const float cxs = K.c[2 * o + 1] * K.inv_dx;
-                    put(i0 + 0, cxs * PX(i0 + 0));
-                    put(i0 + 1, -cxs * NX(i0 + 1));
-                    put(i0 + 2, -cxs * NX(i0 + 2));
-                    put(i0 + 3, cxs * PX(i0 + 3));
-                }
-#undef PX
-#undef NX
-                if (act1)
-                    *reinterpret_cast<float2*>(out + 16 * K.plane + g) = ln.v;
-                else if (act0)
-                    out[16 * K.plane + g] = ln.x();
+                const float ln = clamp01(ad(lam, fm(mu(-E.dtdx, ux), nnd(12, lam, negative(ux)), dlam)));
+                if (!fixed) lam = ln;
             }
-            __syncthreads(); // the staging buffer and macro row are reused
-            cb ^= 1;
+            if (mine) {
+                float* dst = out + ip.off + x;
+#pragma unroll
+                for (int i = 0; i < 16; i++) dst[i * plane] = f[i];
+                dst[16 * plane] = lam;
+            }
         }
-        cp_wait<0>();
-        if (__syncthreads_or(bad) && tid == 0) atomicOr(&b.ctr->status, 1);
-        bad = 0;
+        done += m;
+        if (__syncthreads_or(bad) && t == 0) atomicOr(&b.ctr->status, 1);
         if (!grid_barrier(b, expected)) return;
-        if (blockIdx.x == 0 && tid == 0) b.ctr->step += 1;
+        if (blockIdx.x == 0 && t == 0) b.ctr->step += m;
     }
 }
 
@@ -301,7 +217,11 @@ cudaError_t batch_launch_t(const ModelConst<float>& K, const BatchLaunch& b, int
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, batch_kernel<REC, BT>, K, b);
+    StepConst<float> E;
+    step_const(K, &E);
+    E.c8 = E.c9 = 1.f; // A8c and A9c are the instances'
+    E.a_hat = 1;
+    return cudaLaunchKernelEx(&cfg, batch_kernel<REC, BT>, K, E, b);
 }
 
 constexpr int TI_THREADS = 256;
@@ -391,25 +311,25 @@ cudaError_t launch_tne_instances(int precision, const ModelConst<double>& Kd, co
     return cudaGetLastError();
 }
 
-int batch_segment(int block_threads) { return 2 * block_threads; }
+int batch_segment(int block_threads) { return block_threads - 4 * BATCH_STEPS; }
+int batch_phases(int nsteps) { return (nsteps + BATCH_STEPS - 1) / BATCH_STEPS; }
 
 int batch_max_blocks(int recovery, int block_threads)
 {
-    if (block_threads == 64)
-        return recovery == 1 ? batch_max_blocks_per_sm<1, 64>() : batch_max_blocks_per_sm<0, 64>();
     if (block_threads == 128)
-        return recovery == 1 ? batch_max_blocks_per_sm<1, 128>() : batch_max_blocks_per_sm<0, 128>();
+        return recovery == 1 ? batch_max_blocks_per_sm<2, 128>() : batch_max_blocks_per_sm<0, 128>();
+    if (block_threads == 64)
+        return recovery == 1 ? batch_max_blocks_per_sm<2, 64>() : batch_max_blocks_per_sm<0, 64>();
     return -1;
 }
 
 cudaError_t launch_batch(int recovery, int block_threads, const ModelConst<float>& K,
                          const BatchLaunch& b, int grid, cudaStream_t s)
 {
-    if (block_threads == 64)
-        return recovery == 1 ? batch_launch_t<1, 64>(K, b, grid, s) : batch_launch_t<0, 64>(K, b, grid, s);
     if (block_threads == 128)
-        return recovery == 1 ? batch_launch_t<1, 128>(K, b, grid, s)
-                             : batch_launch_t<0, 128>(K, b, grid, s);
+        return recovery == 1 ? batch_launch_t<2, 128>(K, b, grid, s) : batch_launch_t<0, 128>(K, b, grid, s);
+    if (block_threads == 64)
+        return recovery == 1 ? batch_launch_t<2, 64>(K, b, grid, s) : batch_launch_t<0, 64>(K, b, grid, s);
     return cudaErrorInvalidValue;
 }
 

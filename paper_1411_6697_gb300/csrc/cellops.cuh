@@ -397,8 +397,9 @@ __device__ __forceinline__ S1 s_norm(S1 a)
     return {s, __fsub_rn(a.lo, __fsub_rn(s, a.hi))};
 }
 
-// rho, u, T of one FP32 cell: exact conserved sums, then FP64 (REC = 0) or double-float
-// (REC = 1); ig = T > T_ig in that precision, ok = rho, T > 0 and everything finite
+// rho, u, T of one FP32 cell: exact conserved sums, then FP64 (REC = 0) or double-float (REC = 1
+// normalised throughout, REC = 2 one correction per quotient); ig = T > T_ig in that precision,
+// ok = rho, T > 0 and everything finite
 template <int REC>
 __device__ __forceinline__ void recover32(const ModelConst<float>& K, const float* f, float& rho,
                                           float& ux, float& uy, float& T, bool& ig, bool& ok)
@@ -437,6 +438,29 @@ __device__ __forceinline__ void recover32(const ModelConst<float>& K, const floa
                                    s_add(s_mul(AY[2], K.cdh[1], K.cdl[1]), s_mul(AY[3], K.cdh[3], K.cdl[3]))));
         const S1 m4 = s_norm(s_add(s_add(s_mul(P[0], K.wdh[0], K.wdl[0]), s_mul(P[1], K.wdh[2], K.wdl[2])),
                                    s_add(s_mul(E[0], K.wdh[1], K.wdl[1]), s_mul(E[1], K.wdh[3], K.wdl[3]))));
+        if constexpr (REC == 2) { // quotients of the sums with one correction, as recover_pair_df
+            const float q = rcp_approx(m1.hi);
+            auto quot = [&](S1 a) -> S1 {
+                const float x = __fmul_rn(a.hi, q);
+                float e = __fmaf_rn(-m1.hi, x, a.hi);
+                e = __fadd_rn(e, __fmaf_rn(-m1.lo, x, a.lo));
+                return s_norm({x, __fmul_rn(e, q)});
+            };
+            auto sqr = [](S1 a) -> S1 {
+                const float p = __fmul_rn(a.hi, a.hi);
+                return s_norm({p, __fmaf_rn(__fmul_rn(2.f, a.hi), a.lo, __fmaf_rn(a.hi, a.hi, -p))});
+            };
+            const S1 vx = quot(m2), vy = quot(m3), e = quot(m4);
+            const S1 w = s_norm(s_add(sqr(vx), sqr(vy)));
+            const S1 tt = s_norm(s_mul(s_norm(s_sub(e, w)), K.idh, K.idl));
+            rho = m1.hi;
+            ux = vx.hi;
+            uy = vy.hi;
+            T = tt.hi;
+            ig = T > K.tigh || (T == K.tigh && tt.lo > K.tigl);
+            ok = rho > 0.f && T > 0.f && T <= FLT_MAX && fabsf(ux) <= FLT_MAX && fabsf(uy) <= FLT_MAX;
+            return;
+        }
         double u, v, t;
         const double r = df_to_f64_fast(m1.hi, m1.lo);
         recover_one_f64_fast(m1.hi, m1.lo, r, df_to_f64_fast(m2.hi, m2.lo), df_to_f64_fast(m3.hi, m3.lo),

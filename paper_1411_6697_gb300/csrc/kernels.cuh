@@ -107,7 +107,8 @@ struct BatchLaunch {
     int phantom_blocks;  // > 0 only to test the bounded barrier wait
     long long wait_ns;   // bound of each barrier wait
 };
-int batch_segment(int block_threads);
+int batch_segment(int block_threads); // cells of a work item
+int batch_phases(int nsteps);         // passes over the state (buffer swaps) of nsteps steps
 int batch_max_blocks(int recovery, int block_threads);
 cudaError_t launch_batch(int recovery, int block_threads, const ModelConst<float>& K,
                          const BatchLaunch& b, int grid, cudaStream_t s);
