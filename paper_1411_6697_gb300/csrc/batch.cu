@@ -10,12 +10,13 @@
 // phases; its wait is bounded in time and reports a timeout through the status word instead of
 // hanging. The launch is cooperative, so all blocks are resident.
 //
-// What bounds it: instruction issue and the FP64 unit of the recovery (13 of its instructions a
+// What bounds it: instruction issue and the FP64 unit of the recovery (8 of its instructions a
 // warp and step, 64 cycles each). Two steps per pass took half the state's traffic and half the
 // barriers off; one cell per thread instead of a pair leaves registers for six blocks of 128 on
 // an SM. 512 detonations, 7.95 M cells, ms per step: one step per pass and a pair of cells per
 // thread 0.430; one cell and two steps 0.330 (four 0.361: the shared edges grow; five or eight
-// blocks an SM 0.356, 0.333).
+// blocks an SM 0.356, 0.333); with the pairs joined on the integer pipe (pair_to_f64) 0.315 (one
+// step 0.367, three 0.329).
 #include <float.h>
 #include <stdint.h>
 

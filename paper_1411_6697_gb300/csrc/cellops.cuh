@@ -462,9 +462,9 @@ __device__ __forceinline__ void recover32(const ModelConst<float>& K, const floa
             return;
         }
         double u, v, t;
-        const double r = df_to_f64_fast(m1.hi, m1.lo);
-        recover_one_f64_fast(m1.hi, m1.lo, r, df_to_f64_fast(m2.hi, m2.lo), df_to_f64_fast(m3.hi, m3.lo),
-                             df_to_f64_fast(m4.hi, m4.lo), K.inv_DId, u, v, t);
+        const double r = pair_to_f64(m1.hi, m1.lo);
+        recover_one_f64_fast(m1.hi, m1.lo, r, pair_to_f64(m2.hi, m2.lo), pair_to_f64(m3.hi, m3.lo),
+                             pair_to_f64(m4.hi, m4.lo), K.inv_DId, u, v, t);
         rho = m1.hi;
         ux = d2f_fast(u);
         uy = d2f_fast(v);

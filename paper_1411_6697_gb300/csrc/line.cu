@@ -13,12 +13,12 @@
 // everything that can leave that unit does (cellops.cuh); each difference of neighbouring
 // cells is formed once and exchanged: 298 FP64 instructions per warp and step (ncu, 16384-cell
 // detonation). FP32: the latency of one warp's chain of about 900 instructions; the conserved
-// sums are exact double-floats, which keeps all but 14 FP64 instructions off that unit.
+// sums are exact double-floats, which keeps all but 8 FP64 instructions off that unit.
 //
 // Measured per step, against one launch per step of a tile kernel with the plain formulas
 // (every stencil's differences, FP64 minmod and FP64 sums of an FP32 state): Sod tube of 400
 // cells FP64 29.8 -> 11.7 us (6.8 with four warps to a window, below); detonation of 16384 cells
-// FP32 13.3 -> 2.1 us, FP64 with records at every step 58.9 -> 24.9 us.
+// FP32 13.3 -> 2.0 us, FP64 with records at every step 58.9 -> 24.9 us.
 //
 // Boundaries: lanes past a zero-gradient end are read through the index of the end cell,
 // lanes past a Dirichlet end hold the side's equilibrium, and on a periodic grid every lane

@@ -277,6 +277,20 @@ __device__ __forceinline__ float d2f_fast(double x)
 }
 __device__ __forceinline__ double df_to_f64_fast(float hi, float lo) { return f2d_fast(hi) + f2d_fast(lo); }
 
+// hi + lo rounded to binary64 on the integer pipe, for normalised pairs (|lo| at most a unit in
+// the last place of hi, the reciprocal seed's 2^-22 hi included): lo in units of the last place
+// of hi's binary64 image is added to that image as an integer. Below a power of two those units
+// halve. An FP64 addition would hold the FP64 unit for 64 cycles a warp.
+__device__ __forceinline__ double pair_to_f64(float hi, float lo)
+{
+    const unsigned hb = __float_as_uint(hi);
+    const unsigned e = (306u << 23) - (hb & 0x7f800000u), top = 254u << 23; // 2^(52 - exponent of hi)
+    const float l = __uint_as_float(__float_as_uint(lo) ^ (hb & 0x80000000u));
+    int k = __float2int_rn(l * __uint_as_float(e < top ? e : top));
+    if ((hb & 0x7fffffu) == 0u && k < 0) k += k;
+    return __longlong_as_double(__double_as_longlong(f2d_fast(hi)) + k);
+}
+
 // FP64 recovery of one cell with fewer FP64 operations: 1/m1 seeded by a double-float
 // reciprocal formed on the FP32 pipes (the FP32 estimate r corrected by r (1 - m1 r),
 // about 46 correct bits) and finished by one FP64 Newton step; u = m2 q, v = m3 q; and
@@ -287,7 +301,7 @@ __device__ __forceinline__ void recover_one_f64_fast(float m1h, float m1l, doubl
 {
     const float r = rcp_approx(m1h);
     const float e = fmaf(-m1h, r, 1.0f) - m1l * r; // 1 - m1 r to FP32 accuracy
-    double q = f2d_fast(r) + f2d_fast(r * e);
+    double q = pair_to_f64(r, r * e);
     q = ::fma(q, ::fma(-m1, q, 1.0), q);
     u = m2 * q;
     v = m3 * q;
@@ -308,13 +322,13 @@ __device__ __forceinline__ void recover_pair_fast(const V2* f, const DfConst& C,
         D2 m1, m2, m3, m4;
         conserved_pair_u(f, C, m1, m2, m3, m4);
         double u0, v0, t0, u1, v1, t1;
-        const double r0 = df_to_f64_fast(m1.hi.x(), m1.lo.x());
-        const double r1 = df_to_f64_fast(m1.hi.y(), m1.lo.y());
-        recover_one_f64_fast(m1.hi.x(), m1.lo.x(), r0, df_to_f64_fast(m2.hi.x(), m2.lo.x()),
-                             df_to_f64_fast(m3.hi.x(), m3.lo.x()), df_to_f64_fast(m4.hi.x(), m4.lo.x()),
+        const double r0 = pair_to_f64(m1.hi.x(), m1.lo.x());
+        const double r1 = pair_to_f64(m1.hi.y(), m1.lo.y());
+        recover_one_f64_fast(m1.hi.x(), m1.lo.x(), r0, pair_to_f64(m2.hi.x(), m2.lo.x()),
+                             pair_to_f64(m3.hi.x(), m3.lo.x()), pair_to_f64(m4.hi.x(), m4.lo.x()),
                              K.inv_DId, u0, v0, t0);
-        recover_one_f64_fast(m1.hi.y(), m1.lo.y(), r1, df_to_f64_fast(m2.hi.y(), m2.lo.y()),
-                             df_to_f64_fast(m3.hi.y(), m3.lo.y()), df_to_f64_fast(m4.hi.y(), m4.lo.y()),
+        recover_one_f64_fast(m1.hi.y(), m1.lo.y(), r1, pair_to_f64(m2.hi.y(), m2.lo.y()),
+                             pair_to_f64(m3.hi.y(), m3.lo.y()), pair_to_f64(m4.hi.y(), m4.lo.y()),
                              K.inv_DId, u1, v1, t1);
         rho = m1.hi; // the exact sum rounded to FP32
         ux = V2(d2f_fast(u0), d2f_fast(u1));
