@@ -183,10 +183,10 @@ __global__ void __launch_bounds__(LINE_THREADS)
             if constexpr (sizeof(R) == 8) { // two FMAs
                 if (k >= 0) W[i] = fm(c, nnd(k, f[i], k >= 6), W[i]);
                 nf[i] = fm(K.dt, W[i], f[i]);
-            } else { // the increment first: one rounding at the size of f
-                W[i] = mu(K.dt, W[i]);
-                if (k >= 0) W[i] = fm(c, nnd(k, f[i], k >= 6), W[i]);
-                nf[i] = ad(f[i], W[i]);
+            } else if (k >= 0) { // the increment first: one rounding at the size of f
+                nf[i] = ad(f[i], fm(c, nnd(k, f[i], k >= 6), mu(K.dt, W[i])));
+            } else {
+                nf[i] = fm(K.dt, W[i], f[i]);
             }
         }
         nlam = ad(lam, fm(mu(-E.dtdx, ux), nnd(12, lam, negative(ux)), dlam));
