@@ -478,13 +478,13 @@ LinePlan line_plan(int precision, int nx, bool tne)
                                             : (w > 21.0 ? 0.17 * w : 0.85 + 0.131 * w) + 2.0 / steps;
             if (t < t_best) t_best = t, best = {threads, steps, grid, false};
         }
-    // four warps to a window of 32 cells while every window has an SM of its own (400 cells: 6.8
-    // us per step against 11.7; two windows on an SM would share its FP64 unit and take twice as
-    // long for at most twice the cells of one warp per quarter)
+    // four warps to a window of 32 cells while an SM gets two windows at most (us per step, host
+    // clock: 400 cells 7.2 against 11.7, 4200 cells 8.8; two windows, which share the FP64 unit:
+    // 4864 cells 10.2 against 13.0, 8192 cells 11.7 against 14.2; a third would bring it to 14)
     for (int steps = 1; precision == 0 && !tne && steps <= 4; steps *= 2) {
         const int own = 32 - 4 * steps, grid = (nx + own - 1) / own;
-        const double t = 5.0 + 1.5 / steps;
-        if (grid <= sms && t < t_best) t_best = t, best = {128, steps, grid, true};
+        const double t = (grid <= sms ? 6.7 : 9.7) + 2.0 / steps;
+        if (grid <= 2 * sms && t < t_best) t_best = t, best = {128, steps, grid, true};
     }
     return best;
 }
