@@ -105,24 +105,25 @@ __device__ __forceinline__ Fly<R> butterflies(const R* f)
     b.o3 = u01 + u23;
     return b;
 }
-template <typename R>
+// LAST0: the first term is added last (the FP32 1-D step: orbit 0 has the largest coefficients in
+// the usual sets; Sjogreen tube: the pressure 1.14 times the oracle's distance from the exact
+// solution instead of 1.27)
+template <bool LAST0, typename R>
 __device__ __forceinline__ R dot4(const R* c, R w, R x, R y, R z)
 {
-    // FP32: orbit 0, with the largest coefficients in the usual sets, is added last (Sjogreen tube:
-    // the pressure 1.14 times the oracle's distance from the exact solution instead of 1.27)
-    if constexpr (sizeof(R) == 4) return fm(c[0], w, fm(c[1], x, fm(c[2], y, mu(c[3], z))));
+    if constexpr (LAST0) return fm(c[0], w, fm(c[1], x, fm(c[2], y, mu(c[3], z))));
     return fm(c[3], z, fm(c[2], y, fm(c[1], x, mu(c[0], w))));
 }
 
 // Delta_5..16 = f_hat - f_hat^eq, the equilibrium entering as the product of an FMA
 // (m1 = rho, m2 = rho u_x, m3 = rho u_y)
-template <typename R>
+template <bool LAST0 = false, typename R>
 __device__ __forceinline__ void deltas(const ModelConst<R>& K, const StepConst<R>& E, const Fly<R>& b,
                                        R m1, R m2, R m3, R ux, R uy, R ux2, R uy2, R u2, R T, R pT, R* D)
 {
     const R Ta = ad(T, ux2), Tb = ad(T, uy2);
     const R A = fm(E.di2, T, u2), B = fm(R(2), T, A);
-    const R p2 = dot4(E.h2, b.P0, b.P2, b.e1, b.e3), p3 = dot4(E.h3, b.P0, b.P2, b.e1, b.e3);
+    const R p2 = dot4<LAST0>(E.h2, b.P0, b.P2, b.e1, b.e3), p3 = dot4<LAST0>(E.h3, b.P0, b.P2, b.e1, b.e3);
     const R a0 = fm(E.ha[1], b.M2, mu(E.ha[0], b.M0)), a1 = fm(E.ha[3], b.M2, mu(E.ha[2], b.M0));
     D[0] = fm(-m1, Ta, ad(p2, a0));
     D[2] = fm(-m1, Tb, ad(p2, -a0));
@@ -130,12 +131,12 @@ __device__ __forceinline__ void deltas(const ModelConst<R>& K, const StepConst<R
     D[11] = fm(-mu(m3, uy), B, fm(-pT, A, ad(p3, -a1)));
     D[1] = fm(-m2, uy, fm(K.Boo[1], b.o3, mu(K.Boo[0], b.o1)));
     D[10] = fm(-mu(m2, uy), B, fm(K.Boo[3], b.o3, mu(K.Boo[2], b.o1)));
-    D[3] = fm(-m2, A, dot4(K.Bodd + 4, b.ax0, b.ax2, b.ax1, b.ax3));
-    D[5] = fm(-m2, fm(R(2), T, Ta), dot4(K.Bodd + 8, b.ax0, b.ax2, b.ax1, b.ax3));
-    D[7] = fm(-m2, Tb, dot4(K.Bodd + 12, b.ax0, b.ax2, b.ax1, b.ax3));
-    D[4] = fm(-m3, A, dot4(K.Bodd + 4, b.ay0, b.ay2, b.ay1, b.ay3));
-    D[8] = fm(-m3, fm(R(2), T, Tb), dot4(K.Bodd + 8, b.ay0, b.ay2, b.ay1, b.ay3));
-    D[6] = fm(-m3, Ta, dot4(K.Bodd + 12, b.ay0, b.ay2, b.ay1, b.ay3));
+    D[3] = fm(-m2, A, dot4<LAST0>(K.Bodd + 4, b.ax0, b.ax2, b.ax1, b.ax3));
+    D[5] = fm(-m2, fm(R(2), T, Ta), dot4<LAST0>(K.Bodd + 8, b.ax0, b.ax2, b.ax1, b.ax3));
+    D[7] = fm(-m2, Tb, dot4<LAST0>(K.Bodd + 12, b.ax0, b.ax2, b.ax1, b.ax3));
+    D[4] = fm(-m3, A, dot4<LAST0>(K.Bodd + 4, b.ay0, b.ay2, b.ay1, b.ay3));
+    D[8] = fm(-m3, fm(R(2), T, Tb), dot4<LAST0>(K.Bodd + 8, b.ay0, b.ay2, b.ay1, b.ay3));
+    D[6] = fm(-m3, Ta, dot4<LAST0>(K.Bodd + 12, b.ay0, b.ay2, b.ay1, b.ay3));
 }
 
 // W = Omega = M^-1 [-S Delta + A_hat + C_hat] in block form (Omega_hat_1..3 vanish). S: the

@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(LINE_THREADS)
                   R(0), R(0), A8, A9);
         R D[TNE_K], W[16];
         const R pT = mu(m1, T);
-        deltas(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
+        deltas<sizeof(R) == 4>(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
         if (do_tne) {
             R d2 = mu(D[0], D[0]);
             td[t] = D[0];
