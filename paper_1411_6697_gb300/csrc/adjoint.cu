@@ -199,7 +199,7 @@ __global__ void __launch_bounds__(REV_THREADS)
         const double gyx = mu(pub[14 * n + r1] - pub[14 * n + l1], A.gx);
         const double pT = mu(m1, T), rinv = recip64(m1);
         double D[TNE_K];
-        deltas(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
+        deltas<true>(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
         __syncthreads();
 
         // stencil weights: t = -(dt v / 2 dx) fb for f_i, the branches as bits

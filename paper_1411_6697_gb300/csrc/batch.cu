@@ -16,7 +16,8 @@
 // an SM. 512 detonations, 7.95 M cells, ms per step: one step per pass and a pair of cells per
 // thread 0.430; one cell and two steps 0.330 (four 0.361: the shared edges grow; five or eight
 // blocks an SM 0.356, 0.333); with the pairs joined on the integer pipe (pair_to_f64) 0.315 (one
-// step 0.367, three 0.329).
+// step 0.367, three 0.329), with the even moments' equilibria rounded before they are subtracted
+// (deltas, cellops.cuh) 0.322.
 #include <float.h>
 #include <stdint.h>
 
@@ -139,20 +140,20 @@ __global__ void __launch_bounds__(BT, 768 / BT)
                 if (mine && !ok) bad = 1;
                 hot = hot && lam != 1.f;
                 const float m2 = mu(m1, ux), m3 = mu(m1, uy);
-                const float ux2 = mu(ux, ux), uy2 = mu(uy, uy), u2 = ad(ux2, uy2), pT = mu(m1, T);
+                const float ux2 = mu(ux, ux), uy2 = mu(uy, uy), u2 = fm(ux, ux, uy2), pT = mu(m1, T);
 #pragma unroll
                 for (int k = 0; k < BNX; k++) P[k * BT + t] = slot_plane(k) == 16 ? lam : f[slot_plane(k) & 15];
                 P[BNX * BT + t] = ux;
                 P[(BNX + 1) * BT + t] = uy;
                 __syncthreads();
                 float D[TNE_K], W[16], A8, A9;
-                deltas(K, E, fl, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
+                deltas<true>(K, E, fl, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
                 a_hat<false>(E, ux, uy, P[BNX * BT + jp1] - P[BNX * BT + jm1],
                              P[(BNX + 1) * BT + jp1] - P[(BNX + 1) * BT + jm1], 0.f, 0.f, A8, A9);
                 const bool react = __any_sync(0xffffffffu, hot);
                 float dlam = 0.f;
                 if (react && hot) dlam = reaction_increment(lam, mu(par[19], pT), mu(par[20], pT), K.dt);
-                collide(K, E, par, D, m1, m2, m3, ux, uy, u2, T, pT, mu(par[16], A8), mu(par[17], A9), react,
+                collide<true>(K, E, par, D, m1, m2, m3, ux, uy, u2, T, mu(pT, par[16]), mu(pT, par[17]), A8, A9, react,
                         mu(dlam, par[18]), W);
                 auto nnd = [&](int k, float q, bool neg) -> float {
                     const float* r = P + k * BT;
@@ -160,11 +161,11 @@ __global__ void __launch_bounds__(BT, 768 / BT)
                     return neg ? nnd3(q - l, g - q, r[jp2] - g, true) : nnd3(l - r[jm2], q - l, g - q, false);
                 };
 #pragma unroll
-                for (int i = 0; i < 16; i++) { // the increment first: one rounding at the size of f
+                for (int i = 0; i < 16; i++) {
                     const int k = slot_of(i);
-                    float w = mu(K.dt, W[i]);
+                    float w = W[i];
                     if (k >= 0) w = fm(k >= 6 ? E.cdx[i >> 2] : -E.cdx[i >> 2], nnd(k, f[i], k >= 6), w);
-                    if (!fixed) f[i] = ad(f[i], w);
+                    if (!fixed) f[i] = fm(K.dt, w, f[i]);
                 }
                 const float ln = clamp01(ad(lam, fm(mu(-E.dtdx, ux), nnd(12, lam, negative(ux)), dlam)));
                 if (!fixed) lam = ln;

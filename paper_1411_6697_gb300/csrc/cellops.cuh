@@ -5,7 +5,7 @@
 // SM for 64 cycles, whatever its lanes do and whether or not it depends on the one before; an
 // integer or FP32 instruction takes one. So minmod, comparisons, clamps and extremes of FP64
 // values work on their bit patterns, the factors 1/2 of four moments are folded into the
-// matrix, f_hat^eq enters Delta_k as the product of an FMA, the reciprocal is an FP32 seed with
+// matrix, the FP64 f_hat^eq enters Delta_k as the product of an FMA, the reciprocal is an FP32 seed with
 // one third-order correction, and the terms of the reaction and of A_hat are left out of warps
 // and models where they vanish.
 #pragma once
@@ -21,9 +21,9 @@ template <typename R>
 struct StepConst {
     R h2[4], h3[4], ha[4]; // rows of the ES and EA blocks of m_5, m_7, m_14, m_16, halved
     R c8, c9, gx, gy;      // A8c, A9c, 1/(2 dx), 1/(2 dy)
-    R cdx[4], cdy[4];      // c / dx, c / dy of each orbit (FP32: times dt)
+    R cdx[4], cdy[4];      // c / dx, c / dy of each orbit
     R dtdx, dtdy, inv_DI;
-    R di2;                 // D + I + 2
+    R di2, di4;            // D + I + 2, D + I + 4
     int a_hat;             // A_hat does not vanish
 };
 
@@ -105,50 +105,82 @@ __device__ __forceinline__ Fly<R> butterflies(const R* f)
     b.o3 = u01 + u23;
     return b;
 }
-// LAST0: the first term is added last (the FP32 1-D step: orbit 0 has the largest coefficients in
-// the usual sets; Sjogreen tube: the pressure 1.14 times the oracle's distance from the exact
-// solution instead of 1.27)
-template <bool LAST0, typename R>
+template <typename R>
 __device__ __forceinline__ R dot4(const R* c, R w, R x, R y, R z)
 {
-    if constexpr (LAST0) return fm(c[0], w, fm(c[1], x, fm(c[2], y, mu(c[3], z))));
     return fm(c[3], z, fm(c[2], y, fm(c[1], x, mu(c[0], w))));
 }
 
-// Delta_5..16 = f_hat - f_hat^eq, the equilibrium entering as the product of an FMA
-// (m1 = rho, m2 = rho u_x, m3 = rho u_y)
-template <bool LAST0 = false, typename R>
-__device__ __forceinline__ void deltas(const ModelConst<R>& K, const StepConst<R>& E, const Fly<R>& b,
-                                       R m1, R m2, R m3, R ux, R uy, R ux2, R uy2, R u2, R T, R pT, R* D)
+// Delta_5..16 = f_hat - f_hat^eq (m1 = rho, m2 = rho u_x, m3 = rho u_y). FP64: the equilibrium
+// enters as the product of an FMA.
+template <bool>
+__device__ __forceinline__ void deltas(const ModelConst<double>& K, const StepConst<double>& E,
+                                       const Fly<double>& b, double m1, double m2, double m3, double ux, double uy,
+                                       double ux2, double uy2, double u2, double T, double pT, double* D)
 {
-    const R Ta = ad(T, ux2), Tb = ad(T, uy2);
-    const R A = fm(E.di2, T, u2), B = fm(R(2), T, A);
-    const R p2 = dot4<LAST0>(E.h2, b.P0, b.P2, b.e1, b.e3), p3 = dot4<LAST0>(E.h3, b.P0, b.P2, b.e1, b.e3);
-    const R a0 = fm(E.ha[1], b.M2, mu(E.ha[0], b.M0)), a1 = fm(E.ha[3], b.M2, mu(E.ha[2], b.M0));
+    const double Ta = ad(T, ux2), Tb = ad(T, uy2);
+    const double A = fm(E.di2, T, u2), B = fm(2.0, T, A);
+    const double p2 = dot4(E.h2, b.P0, b.P2, b.e1, b.e3), p3 = dot4(E.h3, b.P0, b.P2, b.e1, b.e3);
+    const double a0 = fm(E.ha[1], b.M2, mu(E.ha[0], b.M0)), a1 = fm(E.ha[3], b.M2, mu(E.ha[2], b.M0));
     D[0] = fm(-m1, Ta, ad(p2, a0));
     D[2] = fm(-m1, Tb, ad(p2, -a0));
     D[9] = fm(-mu(m2, ux), B, fm(-pT, A, ad(p3, a1)));
     D[11] = fm(-mu(m3, uy), B, fm(-pT, A, ad(p3, -a1)));
     D[1] = fm(-m2, uy, fm(K.Boo[1], b.o3, mu(K.Boo[0], b.o1)));
     D[10] = fm(-mu(m2, uy), B, fm(K.Boo[3], b.o3, mu(K.Boo[2], b.o1)));
-    D[3] = fm(-m2, A, dot4<LAST0>(K.Bodd + 4, b.ax0, b.ax2, b.ax1, b.ax3));
-    D[5] = fm(-m2, fm(R(2), T, Ta), dot4<LAST0>(K.Bodd + 8, b.ax0, b.ax2, b.ax1, b.ax3));
-    D[7] = fm(-m2, Tb, dot4<LAST0>(K.Bodd + 12, b.ax0, b.ax2, b.ax1, b.ax3));
-    D[4] = fm(-m3, A, dot4<LAST0>(K.Bodd + 4, b.ay0, b.ay2, b.ay1, b.ay3));
-    D[8] = fm(-m3, fm(R(2), T, Tb), dot4<LAST0>(K.Bodd + 8, b.ay0, b.ay2, b.ay1, b.ay3));
-    D[6] = fm(-m3, Ta, dot4<LAST0>(K.Bodd + 12, b.ay0, b.ay2, b.ay1, b.ay3));
+    D[3] = fm(-m2, A, dot4(K.Bodd + 4, b.ax0, b.ax2, b.ax1, b.ax3));
+    D[5] = fm(-m2, fm(2.0, T, Ta), dot4(K.Bodd + 8, b.ax0, b.ax2, b.ax1, b.ax3));
+    D[7] = fm(-m2, Tb, dot4(K.Bodd + 12, b.ax0, b.ax2, b.ax1, b.ax3));
+    D[4] = fm(-m3, A, dot4(K.Bodd + 4, b.ay0, b.ay2, b.ay1, b.ay3));
+    D[8] = fm(-m3, fm(2.0, T, Tb), dot4(K.Bodd + 8, b.ay0, b.ay2, b.ay1, b.ay3));
+    D[6] = fm(-m3, Ta, dot4(K.Bodd + 12, b.ay0, b.ay2, b.ay1, b.ay3));
+}
+// FP32. The equilibria of the even moments are rounded before they are subtracted, like the moments
+// themselves: in a uniform gas the two roundings then mostly cancel and the cell keeps its bits. As
+// products of an FMA they leave the moment's own rounding in Delta, the same one step after step, and
+// the run drifts (mean error of the state over 40 states: Sod tube of 400 cells, 600 steps 3.9e-7,
+// with FMAs throughout 5.7e-7; batched detonations, 100 steps 2.7e-7 and 3.2e-7).
+// FUSE: where products join sums in one FMA (the 1-D steps); without it each is rounded, as the
+// marching kernel's packed pairs do, so that a grid has the same bits in tiles and in strips.
+template <bool FUSE>
+__device__ __forceinline__ float mad(float a, float b, float c) { return FUSE ? fm(a, b, c) : ad(mu(a, b), c); }
+template <bool FUSE>
+__device__ __forceinline__ float less(float m, float a, float b) { return FUSE ? fm(-a, b, m) : sub(m, mu(a, b)); }
+template <bool FUSE>
+__device__ __forceinline__ void deltas(const ModelConst<float>& K, const StepConst<float>& E, const Fly<float>& b,
+                                       float m1, float m2, float m3, float ux, float uy, float ux2, float uy2,
+                                       float u2, float T, float, float* D)
+{
+    const float T3 = mu(3.f, T);
+    const float Ta = mad<FUSE>(ux, ux, T), Tb = mad<FUSE>(uy, uy, T);
+    const float A = mad<FUSE>(E.di2, T, u2), B = mad<FUSE>(E.di4, T, u2), q3 = mu(mu(m1, A), T), xy = mu(m2, uy);
+    const float p2 = dot4(E.h2, b.P0, b.P2, b.e1, b.e3), p3 = dot4(E.h3, b.P0, b.P2, b.e1, b.e3);
+    const float a0 = fm(E.ha[1], b.M2, mu(E.ha[0], b.M0)), a1 = fm(E.ha[3], b.M2, mu(E.ha[2], b.M0));
+    D[0] = sub(ad(p2, a0), mu(m1, Ta));
+    D[2] = sub(ad(p2, -a0), mu(m1, Tb));
+    D[9] = sub(ad(p3, a1), mad<FUSE>(mu(m2, ux), B, q3));
+    D[11] = sub(ad(p3, -a1), mad<FUSE>(mu(m3, uy), B, q3));
+    D[1] = sub(fm(K.Boo[1], b.o3, mu(K.Boo[0], b.o1)), xy);
+    D[10] = less<FUSE>(fm(K.Boo[3], b.o3, mu(K.Boo[2], b.o1)), xy, B);
+    D[3] = less<FUSE>(dot4(K.Bodd + 4, b.ax0, b.ax2, b.ax1, b.ax3), m2, A);
+    D[5] = less<FUSE>(dot4(K.Bodd + 8, b.ax0, b.ax2, b.ax1, b.ax3), m2, mad<FUSE>(ux, ux, T3));
+    D[7] = less<FUSE>(dot4(K.Bodd + 12, b.ax0, b.ax2, b.ax1, b.ax3), m2, Tb);
+    D[4] = less<FUSE>(dot4(K.Bodd + 4, b.ay0, b.ay2, b.ay1, b.ay3), m3, A);
+    D[8] = less<FUSE>(dot4(K.Bodd + 8, b.ay0, b.ay2, b.ay1, b.ay3), m3, mad<FUSE>(uy, uy, T3));
+    D[6] = less<FUSE>(dot4(K.Bodd + 12, b.ay0, b.ay2, b.ay1, b.ay3), m3, Ta);
 }
 
 // W = Omega = M^-1 [-S Delta + A_hat + C_hat] in block form (Omega_hat_1..3 vanish). S: the
-// rates; A8, A9: A_hat_8 and A_hat_9 over rho T; cr: dlambda times the chemical constant,
-// `react` (warp-uniform) if it is nonzero anywhere in the warp.
+// rates; w8 A8, w9 A9: A_hat_8 and A_hat_9 (a_hat); cr: dlambda times the chemical constant,
+// `react` (warp-uniform) if it is nonzero anywhere in the warp. FP64 joins the rows that m_5 and m_7
+// (m_14 and m_16) share with FMAs; FP32 rounds each row, then their sum and difference.
 template <typename R>
 struct Sectors { // M^-1 Omega_hat before the back butterflies
     R es[4], ea[2], ox[4], oy[4], oo[2];
 };
-template <typename R>
+template <bool, typename R>
 __device__ __forceinline__ void sectors(const ModelConst<R>& K, const StepConst<R>& E, const R* S, const R* D, R m1,
-                                        R m2, R m3, R ux, R uy, R u2, R T, R pT, R A8, R A9, bool react,
+                                        R m2, R m3, R ux, R uy, R u2, R T, R w8, R w9, R A8, R A9, bool react,
                                         R cr, Sectors<R>& z)
 {
     R Om[16]; // Omega_hat; the ES and EA sectors already joined (es, ea)
@@ -158,8 +190,8 @@ __device__ __forceinline__ void sectors(const ModelConst<R>& K, const StepConst<
     R es2 = fm(-S[6], D[2], Om[4]), ea0 = fm(S[6], D[2], Om[4]);
     R es3 = fm(-S[15], D[11], Om[13]), ea1 = fm(S[15], D[11], Om[13]);
     if (E.a_hat) { // Eqs. (3)-(4)
-        Om[7] = fm(pT, A8, Om[7]);
-        Om[8] = fm(pT, A9, Om[8]);
+        Om[7] = fm(w8, A8, Om[7]);
+        Om[8] = fm(w9, A9, Om[8]);
     }
     R *pes = z.es, *pea = z.ea, *px = z.ox, *py = z.oy, *po = z.oo, e1 = R(0); // e1: Omega_hat_4
     if (react) { // C_hat = d f_hat^eq / dT cr (Eqs. (19)-(23))
@@ -193,13 +225,55 @@ __device__ __forceinline__ void sectors(const ModelConst<R>& K, const StepConst<
         po[r] = fm(K.Ioo[2 * r + 1], Om[14], mu(K.Ioo[2 * r], Om[5]));
     }
 }
-template <typename R>
+template <bool FUSE>
+__device__ __forceinline__ void sectors(const ModelConst<float>& K, const StepConst<float>& E, const float* S,
+                                        const float* D, float m1, float m2, float m3, float ux, float uy, float u2,
+                                        float T, float w8, float w9, float A8, float A9, bool react, float cr,
+                                        Sectors<float>& z)
+{
+    float Om[16] = {}, e1 = 0.f;
+    if (react) { // C_hat = d f_hat^eq / dT cr
+        const float dA = mad<FUSE>(2.f * E.di2, T, u2), c4 = E.di4, pd = mu(m1, dA);
+        e1 = mu(mu(m1, K.DI), cr);
+        Om[4] = Om[6] = mu(m1, cr);
+        Om[7] = mu(mu(m2, E.di2), cr);
+        Om[8] = mu(mu(m3, E.di2), cr);
+        Om[9] = mu(mu(3.f, m2), cr);
+        Om[10] = mu(m3, cr);
+        Om[11] = mu(m2, cr);
+        Om[12] = mu(mu(3.f, m3), cr);
+        Om[13] = mu(mad<FUSE>(mu(m2, ux), c4, pd), cr);
+        Om[14] = mu(mu(mu(m2, uy), c4), cr);
+        Om[15] = mu(mad<FUSE>(mu(m3, uy), c4, pd), cr);
+    }
+#pragma unroll
+    for (int k = 4; k < 16; k++) Om[k] = fm(-S[k], D[k - 4], Om[k]);
+    if (E.a_hat) {
+        Om[7] = ad(Om[7], mu(w8, A8));
+        Om[8] = ad(Om[8], mu(w9, A9));
+    }
+    const float es2 = ad(Om[4], Om[6]), ea0 = ad(Om[4], -Om[6]), es3 = ad(Om[13], Om[15]), ea1 = ad(Om[13], -Om[15]);
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        z.es[r] = mu(K.Ies[4 * r + 2], es2);
+        if (react) z.es[r] = fm(K.Ies[4 * r + 2], es2, mu(K.Ies[4 * r + 1], e1));
+        z.es[r] = fm(K.Ies[4 * r + 3], es3, z.es[r]);
+        z.ox[r] = fm(K.Iodd[4 * r + 3], Om[11], fm(K.Iodd[4 * r + 2], Om[9], mu(K.Iodd[4 * r + 1], Om[7])));
+        z.oy[r] = fm(K.Iodd[4 * r + 3], Om[10], fm(K.Iodd[4 * r + 2], Om[12], mu(K.Iodd[4 * r + 1], Om[8])));
+    }
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+        z.ea[r] = fm(K.Iea[2 * r + 1], ea1, mu(K.Iea[2 * r], ea0));
+        z.oo[r] = fm(K.Ioo[2 * r + 1], Om[14], mu(K.Ioo[2 * r], Om[5]));
+    }
+}
+template <bool FUSE, typename R>
 __device__ __forceinline__ void collide(const ModelConst<R>& K, const StepConst<R>& E, const R* S, const R* D, R m1,
-                                        R m2, R m3, R ux, R uy, R u2, R T, R pT, R A8, R A9, bool react,
+                                        R m2, R m3, R ux, R uy, R u2, R T, R w8, R w9, R A8, R A9, bool react,
                                         R cr, R* W)
 {
     Sectors<R> z;
-    sectors(K, E, S, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, cr, z);
+    sectors<FUSE>(K, E, S, D, m1, m2, m3, ux, uy, u2, T, w8, w9, A8, A9, react, cr, z);
     const R *pes = z.es, *pea = z.ea, *px = z.ox, *py = z.oy, *po = z.oo;
 #pragma unroll
     for (int c = 0; c < 2; c++) {
@@ -217,24 +291,43 @@ __device__ __forceinline__ void collide(const ModelConst<R>& K, const StepConst<
     }
 }
 
-// A_hat_8 and A_hat_9 over rho T from the differences of u between the right and left
-// (..x) and, on a 2-D grid, the upper and lower (..y) neighbours
-template <bool TWO_D, typename R>
-__device__ __forceinline__ void a_hat(const StepConst<R>& E, R ux, R uy, R dxx, R dyx, R dxy, R dyy, R& A8,
-                                      R& A9)
+// A_hat_8 and A_hat_9 (Eqs. (3)-(4)) as w8 A8 and w9 A9, from the differences of u between the right
+// and left (..x) and, on a 2-D grid, the upper and lower (..y) neighbours. FP64: w8 = w9 = rho T
+// (a_weight).
+template <bool TWO_D>
+__device__ __forceinline__ void a_hat(const StepConst<double>& E, double ux, double uy, double dxx, double dyx,
+                                      double dxy, double dyy, double& A8, double& A9)
 {
-    const R gxx = mu(dxx, E.gx), u4 = mu(R(4), ux), v4 = mu(R(4), uy);
+    const double gxx = mu(dxx, E.gx), u4 = mu(4.0, ux), v4 = mu(4.0, uy);
     if constexpr (TWO_D) {
-        const R gyy = mu(dyy, E.gy), sh = mu(R(2), fm(dxy, E.gy, mu(dyx, E.gx)));
-        const R th = mu(ad(gxx, gyy), E.inv_DI);
+        const double gyy = mu(dyy, E.gy), sh = mu(2.0, fm(dxy, E.gy, mu(dyx, E.gx)));
+        const double th = mu(ad(gxx, gyy), E.inv_DI);
         A8 = mu(E.c8, fm(uy, sh, mu(u4, ad(gxx, -th))));
         A9 = mu(E.c9, fm(ux, sh, mu(v4, ad(gyy, -th))));
     } else {
-        const R sh = mu(R(2), mu(dyx, E.gx)), th = mu(gxx, E.inv_DI);
+        const double sh = mu(2.0, mu(dyx, E.gx)), th = mu(gxx, E.inv_DI);
         A8 = mu(E.c8, fm(uy, sh, mu(u4, ad(gxx, -th))));
         A9 = mu(E.c9, fm(ux, sh, mu(v4, -th)));
     }
 }
+template <bool TWO_D>
+__device__ __forceinline__ void a_hat(const StepConst<float>& E, float ux, float uy, float dxx, float dyx, float dxy,
+                                      float dyy, float& A8, float& A9)
+{
+    const float gxx = mu(dxx, E.gx), x4 = mu(4.f, ux), y4 = mu(4.f, uy);
+    if constexpr (TWO_D) {
+        const float gyy = mu(dyy, E.gy), sh = ad(mu(dyx, E.gx), mu(dxy, E.gy)), th = mu(ad(gxx, gyy), E.inv_DI);
+        A8 = fm(x4, ad(gxx, -th), mu(mu(2.f, uy), sh));
+        A9 = fm(y4, ad(gyy, -th), mu(mu(2.f, ux), sh));
+    } else {
+        const float sh = mu(dyx, E.gx), th = mu(gxx, E.inv_DI);
+        A8 = fm(mu(2.f, uy), sh, mu(x4, fm(dxx, E.gx, -th)));
+        A9 = fm(mu(2.f, ux), sh, mu(y4, -th));
+    }
+}
+// w of a_hat; c: A8c or A9c
+__device__ __forceinline__ double a_weight(double pT, double) { return pT; }
+__device__ __forceinline__ float a_weight(float pT, float c) { return mu(pT, c); }
 
 // The NND flux difference over c from three neighbouring differences around the upwind one:
 // dc + (mm(dc, dr) - mm(dl, dc)) / 2 for v > 0, dc - (mm(dc, dr) - mm(dl, dc)) / 2 for v < 0
@@ -506,9 +599,8 @@ inline void step_const(const ModelConst<R>& K, StepConst<R>* E)
         E->h2[j] = R(0.5) * K.Bes[8 + j];
         E->h3[j] = R(0.5) * K.Bes[12 + j];
         E->ha[j] = R(0.5) * K.Bea[j];
-        const R f = sizeof(R) == 8 ? R(1) : K.dt;
-        E->cdx[j] = f * K.c[j] * K.inv_dx;
-        E->cdy[j] = f * K.c[j] * K.inv_dy;
+        E->cdx[j] = K.c[j] * K.inv_dx;
+        E->cdy[j] = K.c[j] * K.inv_dy;
     }
     E->c8 = K.A8c;
     E->c9 = K.A9c;
@@ -518,6 +610,7 @@ inline void step_const(const ModelConst<R>& K, StepConst<R>* E)
     E->dtdx = K.dt * K.inv_dx;
     E->dtdy = K.dt * K.inv_dy;
     E->di2 = K.DI + R(2);
+    E->di4 = K.DI + R(4);
     E->a_hat = K.A8c != R(0) || K.A9c != R(0);
 }
 

@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(LINE_THREADS)
             m3 = mu(m1, uy);
             ux2 = mu(ux, ux);
             uy2 = mu(uy, uy);
-            u2 = ad(ux2, uy2);
+            u2 = fm(ux, ux, uy2);
         }
 #pragma unroll
         for (int k = 0; k < NX; k++) P[k * n + t] = slot_plane(k) == 16 ? lam : f[slot_plane(k) & 15];
@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(LINE_THREADS)
                   R(0), R(0), A8, A9);
         R D[TNE_K], W[16];
         const R pT = mu(m1, T);
-        deltas<sizeof(R) == 4>(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
+        deltas<true>(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
         if (do_tne) {
             R d2 = mu(D[0], D[0]);
             td[t] = D[0];
@@ -162,7 +162,8 @@ __global__ void __launch_bounds__(LINE_THREADS)
         const bool react = __any_sync(0xffffffffu, hot);
         R dlam = R(0);
         if (react && hot) dlam = reaction_increment(lam, mu(K.omega1, pT), mu(K.omega2, pT), K.dt);
-        collide(K, E, K.S, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, mu(dlam, K.chem), W);
+        collide<true>(K, E, K.S, D, m1, m2, m3, ux, uy, u2, T, a_weight(pT, E.c8), a_weight(pT, E.c9), A8, A9, react,
+                mu(dlam, K.chem), W);
         // NND differences (v > 0 from d_{j-2}, d_{j-1}, d_j; v < 0 from d_{j-1}, d_j, d_{j+1};
         // d_j = q_{j+1} - q_j) and the Euler update; lambda's side by the sign of u_x
         if constexpr (sizeof(R) == 8) __syncthreads();
@@ -180,16 +181,15 @@ __global__ void __launch_bounds__(LINE_THREADS)
         for (int i = 0; i < 16; i++) {
             const int k = slot_of(i);
             const R c = k >= 6 ? E.cdx[i >> 2] : -E.cdx[i >> 2];
-            if constexpr (sizeof(R) == 8) { // two FMAs
-                if (k >= 0) W[i] = fm(c, nnd(k, f[i], k >= 6), W[i]);
-                nf[i] = fm(K.dt, W[i], f[i]);
-            } else if (k >= 0) { // the increment first: one rounding at the size of f
-                nf[i] = ad(f[i], fm(c, nnd(k, f[i], k >= 6), mu(K.dt, W[i])));
-            } else {
-                nf[i] = fm(K.dt, W[i], f[i]);
+            if (k >= 0) { // (FP32: the diagonal orbits' flux is rounded first, as with both axes)
+                const R X = nnd(k, f[i], k >= 6);
+                W[i] = sizeof(R) == 4 && (i >> 2 & 1) ? ad(W[i], mu(c, X)) : fm(c, X, W[i]);
             }
+            nf[i] = fm(K.dt, W[i], f[i]);
         }
-        nlam = ad(lam, fm(mu(-E.dtdx, ux), nnd(12, lam, negative(ux)), dlam));
+        const R X = nnd(12, lam, negative(ux));
+        if constexpr (sizeof(R) == 8) nlam = ad(lam, fm(mu(-E.dtdx, ux), X, dlam));
+        else nlam = ad(fm(-K.dt, mu(mu(ux, X), K.inv_dx), lam), dlam);
         nlam = clamp01(nlam);
         if (do_tne) {
             const int warp = t >> 5;
@@ -338,9 +338,9 @@ __device__ __forceinline__ void split_steps(const ModelConst<double>& K, const S
         }
         // this sector's part of the collision (unused entries and rows fall away)
         double D[TNE_K];
-        deltas(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
+        deltas<true>(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
         Sectors<double> z;
-        sectors(K, E, K.S, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, cr, z);
+        sectors<true>(K, E, K.S, D, m1, m2, m3, ux, uy, u2, T, pT, pT, A8, A9, react, cr, z);
         if constexpr (Q == 0) {
 #pragma unroll
             for (int r = 0; r < 4; r++) tr[r * n + t] = z.es[r];

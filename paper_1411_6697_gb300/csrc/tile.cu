@@ -163,7 +163,7 @@ __global__ void __launch_bounds__(Tile<R>::TT, sizeof(R) == 8 ? 2 : 4)
 
         const R pT = mu(m1, T);
         R D[TNE_K], W[16], A8 = R(0), A9 = R(0);
-        deltas(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
+        deltas<false>(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, pT, D);
         if (do_tne) {
             R d2 = mu(D[0], D[0]);
             td[t] = D[0];
@@ -190,7 +190,8 @@ __global__ void __launch_bounds__(Tile<R>::TT, sizeof(R) == 8 ? 2 : 4)
             const R* v0 = u0 + UH * UW;
             a_hat<true>(E, ux, uy, u0[1] - u0[-1], v0[1] - v0[-1], u0[UW] - u0[-UW], v0[UW] - v0[-UW], A8, A9);
         }
-        collide(K, E, K.S, D, m1, m2, m3, ux, uy, u2, T, pT, A8, A9, react, mu(dlam, K.chem), W);
+        collide<false>(K, E, K.S, D, m1, m2, m3, ux, uy, u2, T, a_weight(pT, E.c8), a_weight(pT, E.c9), A8, A9, react,
+                mu(dlam, K.chem), W);
 
         // NND flux differences of plane i along one axis (stride d), upwind side by `neg`
         auto nnd = [&](const R* q, R q0, int d, bool neg) -> R {
@@ -210,15 +211,25 @@ __global__ void __launch_bounds__(Tile<R>::TT, sizeof(R) == 8 ? 2 : 4)
             const int o = i >> 2, j = i & 3;
             const int sx = (o & 1) ? (j == 0 || j == 3 ? 1 : -1) : (j == 0 ? 1 : (j == 2 ? -1 : 0));
             const int sy = (o & 1) ? (j < 2 ? 1 : -1) : (j == 1 ? 1 : (j == 3 ? -1 : 0));
-            R w = sizeof(R) == 8 ? W[i] : mu(K.dt, W[i]);
-            if (sx != 0) w = fm(sx < 0 ? E.cdx[o] : -E.cdx[o], nnd(s0 + i * PS, f[i], 1, sx < 0), w);
-            if (sy != 0) w = fm(sy < 0 ? E.cdy[o] : -E.cdy[o], nnd(s0 + i * PS, f[i], SW, sy < 0), w);
-            const R v = sizeof(R) == 8 ? fm(K.dt, w, f[i]) : ad(f[i], w);
+            R w = W[i];
+            if constexpr (sizeof(R) == 8) {
+                if (sx != 0) w = fm(sx < 0 ? E.cdx[o] : -E.cdx[o], nnd(s0 + i * PS, f[i], 1, sx < 0), w);
+                if (sy != 0) w = fm(sy < 0 ? E.cdy[o] : -E.cdy[o], nnd(s0 + i * PS, f[i], SW, sy < 0), w);
+            } else { // v . grad f first, as in the marching kernel
+                const R X = sx != 0 ? nnd(s0 + i * PS, f[i], 1, sx < 0) : R(0);
+                const R Y = sy != 0 ? nnd(s0 + i * PS, f[i], SW, sy < 0) : R(0);
+                const R cx = sx < 0 ? -E.cdx[o] : E.cdx[o], cy = sy < 0 ? -E.cdy[o] : E.cdy[o];
+                // (velocity 5 = (-c, c) adds y to x there, the others x to y)
+                w = sub(w, sx == 0 ? mu(cy, Y) : sy == 0 ? mu(cx, X) : j == 1 ? fm(cy, Y, mu(cx, X)) : fm(cx, X, mu(cy, Y)));
+            }
+            const R v = fm(K.dt, w, f[i]);
             if (active) out[i * plane + g] = avg ? fm(wp, prev[i * plane + g], mu(wn, v)) : v;
         }
-        R la = fm(mu(-E.dtdx, ux), nnd_by(s0 + 16 * PS, lam, 1, negative(ux)), dlam);
-        la = fm(mu(-E.dtdy, uy), nnd_by(s0 + 16 * PS, lam, SW, negative(uy)), la);
-        const R ln = clamp01(ad(lam, la));
+        const R lx_ = nnd_by(s0 + 16 * PS, lam, 1, negative(ux)), ly_ = nnd_by(s0 + 16 * PS, lam, SW, negative(uy));
+        R ln;
+        if constexpr (sizeof(R) == 8) ln = ad(lam, fm(mu(-E.dtdy, uy), ly_, fm(mu(-E.dtdx, ux), lx_, dlam)));
+        else ln = ad(fm(-K.dt, fm(mu(ux, K.inv_dx), lx_, mu(mu(uy, K.inv_dy), ly_)), lam), dlam);
+        ln = clamp01(ln);
         if (active) out[16 * plane + g] = avg ? fm(wp, prev[16 * plane + g], mu(wn, ln)) : ln;
     }
 
