@@ -554,12 +554,13 @@ __device__ __forceinline__ Eq24<R> eq24(const Model<R>& K, R rho, R ux, R uy, R 
     e.T = T;
     e.m2 = mu(rho, ux);
     e.m3 = mu(rho, uy);
+    constexpr bool F4 = sizeof(R) == 4; // each of u^2, T + u^2, (D+I+4) T + u^2 rounded once
     const R ux2 = mu(ux, ux), uy2 = mu(uy, uy), I3 = mu(R(3), K.I_r);
-    e.u2 = ad(ux2, uy2);
-    e.Ta = ad(T, ux2);
-    e.Tb = ad(T, uy2);
+    e.u2 = F4 ? fm(ux, ux, uy2) : ad(ux2, uy2);
+    e.Ta = F4 ? fm(ux, ux, T) : ad(T, ux2);
+    e.Tb = F4 ? fm(uy, uy, T) : ad(T, uy2);
     e.A = fm(ad(K.DI_r, R(2)), T, e.u2);
-    e.B = fm(R(2), T, e.A);
+    e.B = F4 ? fm(ad(K.DI_r, R(4)), T, e.u2) : fm(R(2), T, e.A);
     e.pT = mu(rho, T);
     e.IT = mu(K.I_r, T);
     e.rIT = mu(rho, e.IT);
@@ -568,31 +569,43 @@ __device__ __forceinline__ Eq24<R> eq24(const Model<R>& K, R rho, R ux, R uy, R 
     e.H = fm(ad(R(2), I3), T, e.u2);
     return e;
 }
-// f_hat^eq of moment k (0-based), and h - f_hat^eq with the last product inside an FMA
+// h - a b of a moment h and its equilibrium: FP64 one FMA, FP32 the product rounded like the moment
+// (deltas, cellops.cuh)
+__device__ __forceinline__ double less(double h, double a, double b) { return fm(-a, b, h); }
+__device__ __forceinline__ float less(float h, float a, float b) { return sub(h, mu(a, b)); }
+// h - (m1 A T + a B) and 3 T + u^2
+__device__ __forceinline__ double less4(const Eq24<double>& e, double h, double a) { return fm(-a, e.B, fm(-e.pT, e.A, h)); }
+__device__ __forceinline__ float less4(const Eq24<float>& e, float h, float a)
+{
+    return sub(h, fm(mu(e.m1, e.A), e.T, mu(a, e.B)));
+}
+__device__ __forceinline__ double three(double T, double Ta, double) { return fm(2.0, T, Ta); }
+__device__ __forceinline__ float three(float T, float, float u) { return fm(3.f, T, mu(u, u)); }
+// h - f_hat^eq of moment k (0-based)
 template <typename R>
 __device__ __forceinline__ R minus_eq(const Eq24<R>& e, int k, R h)
 {
     switch (k) {
-    case 4: return fm(-e.m1, e.Ta, h);
-    case 5: return fm(-e.m2, e.uy, h);
-    case 6: return fm(-e.m1, e.Tb, h);
-    case 7: return fm(-e.m2, e.A, h);
-    case 8: return fm(-e.m3, e.A, h);
-    case 9: return fm(-e.m2, fm(R(2), e.T, e.Ta), h);
-    case 10: return fm(-e.m3, e.Ta, h);
-    case 11: return fm(-e.m2, e.Tb, h);
-    case 12: return fm(-e.m3, fm(R(2), e.T, e.Tb), h);
-    case 13: return fm(-mu(e.m2, e.ux), e.B, fm(-e.pT, e.A, h));
-    case 14: return fm(-mu(e.m2, e.uy), e.B, h);
-    case 15: return fm(-mu(e.m3, e.uy), e.B, fm(-e.pT, e.A, h));
-    case 16: return fm(-e.rIT, e.Ta, h);
-    case 17: return fm(-mu(e.m2, e.uy), e.IT, h);
-    case 18: return fm(-e.rIT, e.Tb, h);
-    case 19: return fm(-e.rIT, e.H, h);
-    case 20: return fm(-e.m2, e.C, h);
-    case 21: return fm(-e.m3, e.C, h);
-    case 22: return fm(-e.m2, e.G, h);
-    default: return fm(-e.m3, e.G, h);
+    case 4: return less(h, e.m1, e.Ta);
+    case 5: return less(h, e.m2, e.uy);
+    case 6: return less(h, e.m1, e.Tb);
+    case 7: return less(h, e.m2, e.A);
+    case 8: return less(h, e.m3, e.A);
+    case 9: return less(h, e.m2, three(e.T, e.Ta, e.ux));
+    case 10: return less(h, e.m3, e.Ta);
+    case 11: return less(h, e.m2, e.Tb);
+    case 12: return less(h, e.m3, three(e.T, e.Tb, e.uy));
+    case 13: return less4(e, h, mu(e.m2, e.ux));
+    case 14: return less(h, mu(e.m2, e.uy), e.B);
+    case 15: return less4(e, h, mu(e.m3, e.uy));
+    case 16: return less(h, e.rIT, e.Ta);
+    case 17: return less(h, mu(e.m2, e.uy), e.IT);
+    case 18: return less(h, e.rIT, e.Tb);
+    case 19: return less(h, e.rIT, e.H);
+    case 20: return less(h, e.m2, e.C);
+    case 21: return less(h, e.m3, e.C);
+    case 22: return less(h, e.m2, e.G);
+    default: return less(h, e.m3, e.G);
     }
 }
 
