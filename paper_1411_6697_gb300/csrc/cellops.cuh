@@ -45,12 +45,18 @@ __device__ __forceinline__ double unorder64(long long k)
 {
     return __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
 }
-// 1/x: FP32 estimate (22 bits), then q + q (e + e^2), e = 1 - x q
+// 1/x: FP32 estimate (22 bits), then q + q (e + e^2), e = 1 - x q, of x scaled to [1, 2) by its
+// exponent field; the exponent goes back into the result on the integer pipe. NaN where the result
+// or x is not a normal number (x zero, subnormal, from 2^1022 on or not finite), so that the tests
+// on T see it.
 __device__ __forceinline__ double recip64(double x)
 {
-    const double q = f2d_fast(rcp_approx(d2f_fast(x)));
-    const double e = __fma_rn(-x, q, 1.0);
-    return __fma_rn(q, __fma_rn(e, e, e), q);
+    const int hi = __double2hiint(x), e2 = hi & 0x7ff00000;
+    const double s = __hiloint2double(hi - e2 + 0x3ff00000, __double2loint(x));
+    const double q = f2d_fast(rcp_approx(d2f_fast(s)));
+    const double e = __fma_rn(-s, q, 1.0), r = __fma_rn(q, __fma_rn(e, e, e), q);
+    const bool normal = (unsigned)(e2 - 0x00100000) < 0x7fc00000u;
+    return __hiloint2double(normal ? __double2hiint(r) + 0x3ff00000 - e2 : 0x7ff80000, __double2loint(r));
 }
 
 // Rounded operations that the compiler must not merge: every path through the step then
