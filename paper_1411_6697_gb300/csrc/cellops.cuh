@@ -146,8 +146,7 @@ __device__ __forceinline__ void deltas(const ModelConst<double>& K, const StepCo
 // products of an FMA they leave the moment's own rounding in Delta, the same one step after step, and
 // the run drifts (mean error of the state over 40 states: Sod tube of 400 cells, 600 steps 3.9e-7,
 // with FMAs throughout 5.7e-7; batched detonations, 100 steps 2.7e-7 and 3.2e-7).
-// FUSE: where products join sums in one FMA (the 1-D steps); without it each is rounded, as the
-// marching kernel's packed pairs do, so that a grid has the same bits in tiles and in strips.
+// FUSE: where products join sums in one FMA (the 1-D steps); without it each is rounded (the tiles).
 template <bool FUSE>
 __device__ __forceinline__ float mad(float a, float b, float c) { return FUSE ? fm(a, b, c) : ad(mu(a, b), c); }
 template <bool FUSE>
@@ -578,14 +577,18 @@ __device__ __forceinline__ void recover32(const ModelConst<float>& K, const floa
     }
 }
 
-// rho, u, T of one FP64 cell from its butterflies (Eqs. (5)-(7)); ok: rho, T > 0 and finite
+// rho, u, T of one FP64 cell from its butterflies (Eqs. (5)-(7)); ok: rho, T > 0 and finite.
+// AXIS_FIRST: the momenta of the axis orbits are added before the diagonal ones (the 2-D step), else
+// in the orbits' order
+template <bool AXIS_FIRST = false>
 __device__ __forceinline__ void recover64(const ModelConst<double>& K, const Fly<double>& b, double& m1,
                                           double& m2, double& m3, double& ux, double& uy, double& ux2,
                                           double& uy2, double& u2, double& T, bool& ok)
 {
     m1 = (b.P0 + b.P2) + (b.e1 + b.e3);
-    m2 = fm(K.cd[3], b.ax3, fm(K.cd[2], b.ax2, fm(K.cd[1], b.ax1, mu(K.cd[0], b.ax0))));
-    m3 = fm(K.cd[3], b.ay3, fm(K.cd[2], b.ay2, fm(K.cd[1], b.ay1, mu(K.cd[0], b.ay0))));
+    constexpr int s = AXIS_FIRST ? 2 : 1, t = 3 - s; // the second and third orbit
+    m2 = fm(K.cd[3], b.ax3, fm(K.cd[t], t == 1 ? b.ax1 : b.ax2, fm(K.cd[s], s == 1 ? b.ax1 : b.ax2, mu(K.cd[0], b.ax0))));
+    m3 = fm(K.cd[3], b.ay3, fm(K.cd[t], t == 1 ? b.ay1 : b.ay2, fm(K.cd[s], s == 1 ? b.ay1 : b.ay2, mu(K.cd[0], b.ay0))));
     const double m4 = fm(K.wd[3], b.e3, fm(K.wd[1], b.e1, fm(K.wd[2], b.P2, mu(K.wd[0], b.P0))));
     const double q = recip64(m1);
     ux = mu(m2, q);

@@ -40,17 +40,17 @@ struct Tile {
     }
 };
 
-// u of one cell from its 16 values at stride PS (the rim): FP64, or plain FP32
+// u of a cell of the rim from its 16 values at stride PS. FP64: by the formulas of the tile's own
+// cells (what T takes falls away), so a velocity has the same bits in the tile and in its neighbours'
+// rims and grad u of a uniform flow vanishes at tile edges too. FP32: plain FP32, as the marching
+// kernel's strips have it at their sides; the exact sums take 3 % of a step (300 x 100).
 __device__ __forceinline__ void rim_u(const ModelConst<double>& K, const double* s, double& ux, double& uy)
 {
-    constexpr int PS = Tile<double>::PS;
-    double f[16];
+    double f[16], m1, m2, m3, ux2, uy2, u2, T;
+    bool ok;
 #pragma unroll
-    for (int i = 0; i < 16; i++) f[i] = s[i * PS];
-    const Fly<double> b = butterflies(f);
-    const double q = recip64((b.P0 + b.P2) + (b.e1 + b.e3));
-    ux = mu(fm(K.cd[3], b.ax3, fm(K.cd[1], b.ax1, fm(K.cd[2], b.ax2, mu(K.cd[0], b.ax0)))), q);
-    uy = mu(fm(K.cd[3], b.ay3, fm(K.cd[1], b.ay1, fm(K.cd[2], b.ay2, mu(K.cd[0], b.ay0)))), q);
+    for (int i = 0; i < 16; i++) f[i] = s[i * Tile<double>::PS];
+    recover64<true>(K, butterflies(f), m1, m2, m3, ux, uy, ux2, uy2, u2, T, ok);
 }
 __device__ __forceinline__ void rim_u(const ModelConst<float>& K, const float* s, float& ux, float& uy)
 {
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(Tile<R>::TT, sizeof(R) == 8 ? 2 : 4)
         if (y < ny) { // whole warps past the last row have nothing to do
             b = butterflies(f);
             if constexpr (sizeof(R) == 8) {
-                recover64(K, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, ok);
+                recover64<true>(K, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, ok);
                 hot = dbits(T) > dbits(K.T_igd) && dbits(lam) != dbits(1.0);
             } else {
                 recover32<REC>(K, f, m1, ux, uy, T, hot, ok);
@@ -215,11 +215,10 @@ __global__ void __launch_bounds__(Tile<R>::TT, sizeof(R) == 8 ? 2 : 4)
             if constexpr (sizeof(R) == 8) {
                 if (sx != 0) w = fm(sx < 0 ? E.cdx[o] : -E.cdx[o], nnd(s0 + i * PS, f[i], 1, sx < 0), w);
                 if (sy != 0) w = fm(sy < 0 ? E.cdy[o] : -E.cdy[o], nnd(s0 + i * PS, f[i], SW, sy < 0), w);
-            } else { // v . grad f first, as in the marching kernel
+            } else { // v . grad f first
                 const R X = sx != 0 ? nnd(s0 + i * PS, f[i], 1, sx < 0) : R(0);
                 const R Y = sy != 0 ? nnd(s0 + i * PS, f[i], SW, sy < 0) : R(0);
                 const R cx = sx < 0 ? -E.cdx[o] : E.cdx[o], cy = sy < 0 ? -E.cdy[o] : E.cdy[o];
-                // (velocity 5 = (-c, c) adds y to x there, the others x to y)
                 w = sub(w, sx == 0 ? mu(cy, Y) : sy == 0 ? mu(cx, X) : j == 1 ? fm(cy, Y, mu(cx, X)) : fm(cx, X, mu(cy, Y)));
             }
             const R v = fm(K.dt, w, f[i]);
