@@ -791,7 +791,7 @@ lbkm_status lbkm_get_state(lbkm_t h, void* dst, int on_device)
     if (!h || !dst) return LBKM_EINVAL;
     if (!h->initialized) return fail(h, LBKM_ESTATE, "lbkm_get_state before lbkm_init_fields");
     const size_t row = (size_t)h->nx * h->elem, plane = row * h->ny;
-    if (on_device && can_pack((int)h->elem, dst)) {
+    if (on_device && can_pack((int)h->elem, h->buf[h->cur], dst)) {
         CUDA_TRY(h, launch_pack((int)h->elem, NPLANE, h->buf[h->cur], (int64_t)h->plane_elems, h->pitch, h->nx,
                                 h->ny, dst, h->host_steps, h->stream));
         return check_status(h);

@@ -2082,7 +2082,7 @@ lbkm_status lbkm24_get_state(lbkm24_t h, void* dst, int on_device)
     if (!h || !dst) return LBKM_EINVAL;
     if (!h->initialized) return fail(h, LBKM_ESTATE, "lbkm24_get_state before init_fields");
     const size_t row = (size_t)h->p.nx * h->elem, plane = row * h->p.ny;
-    if (on_device && lbk::can_pack((int)h->elem, dst)) {
+    if (on_device && lbk::can_pack((int)h->elem, h->buf[h->cur], dst)) {
         TRY24(h, lbk::launch_pack((int)h->elem, NP, h->buf[h->cur], (int64_t)h->plane_elems, h->pitch, h->p.nx,
                                   h->p.ny, dst, h->host_steps, h->stream));
         return check(h);

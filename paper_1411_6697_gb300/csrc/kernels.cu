@@ -291,18 +291,20 @@ __global__ void __launch_bounds__(256)
 // each (FP32 shock reflection, 300 x 100: 64 steps and a snapshot took 0.80 ms, now 0.71; a copy of
 // its 2 MB, 8 us). 16-byte vectors where the row length and dst allow them (the pitch always
 // does), elements otherwise.
-// Whether launch_pack may write there: memory of the current device, aligned to an element. Memory
-// of another device or of the host is left to the copies, which need no peer access.
-bool can_pack(int elem, const void* dst)
+// Whether launch_pack may write there: memory of the state's device, aligned to an element, that
+// device being the current one (a kernel launches on the stream of no other). Memory of another
+// device or of the host, or another current device, is left to the copies, which need no peer access.
+bool can_pack(int elem, const void* state, const void* dst)
 {
-    cudaPointerAttributes at;
+    cudaPointerAttributes to, from;
     int dev = -1;
-    if (reinterpret_cast<uintptr_t>(dst) % elem) return false;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&at, dst) != cudaSuccess) {
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaPointerGetAttributes(&to, dst) != cudaSuccess ||
+        cudaPointerGetAttributes(&from, state) != cudaSuccess) {
         cudaGetLastError();
         return false;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == dev;
+    return pack_there(elem, reinterpret_cast<uintptr_t>(dst), to.type == cudaMemoryTypeDevice, to.device, from.device,
+                      dev);
 }
 
 cudaError_t launch_pack(int elem, int planes, const void* state, int64_t plane_elems, int pitch, int nx,

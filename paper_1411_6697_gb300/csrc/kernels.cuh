@@ -75,7 +75,12 @@ cudaError_t launch_macros(int precision, const ModelConst<double>& Kd, const voi
                           double* lam, cudaStream_t s);
 // A state snapshot on the device: `planes` planes of ny rows of nx elements (4 or 8 bytes) packed
 // into dst, then the step counter; for the destinations that can_pack accepts.
-bool can_pack(int elem, const void* dst);
+bool can_pack(int elem, const void* state, const void* dst);
+// the rule itself: devices of the state, of dst and the current one, and dst's alignment
+inline bool pack_there(int elem, uintptr_t dst, bool device_memory, int dst_dev, int state_dev, int current)
+{
+    return dst % elem == 0 && device_memory && dst_dev == state_dev && current == state_dev;
+}
 cudaError_t launch_pack(int elem, int planes, const void* state, int64_t plane_elems, int pitch, int nx,
                         int ny, void* dst, int64_t step, cudaStream_t s);
 // TNE fields (optional) and grid-wide record of a state, all FP64.
