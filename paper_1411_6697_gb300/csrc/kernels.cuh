@@ -129,6 +129,26 @@ cudaError_t launch_tne_instances(int precision, const ModelConst<double>& Kd, co
 cudaError_t march_tensor_maps(const void* state, int nx, int ny, int pitch, int64_t plane,
                               TmaDesc* load, TmaDesc* store);
 int march_grid(int mode, int nx, int ny);
+// The strip height of least cost for nsx columns of strips on G resident blocks, at most `cap` (even)
+// rows; `cost` of (strips, rows). Of the heights with the same number of strips the smallest is the
+// cheapest, so only those are tried: about 2 sqrt(ny) of them (every even height up to ny took 1.7 ms
+// a launch at a million rows).
+template <typename Cost>
+inline int march_rows(int ny, int cap, int nsx, Cost cost, int* tried = nullptr)
+{
+    int best_rows = 2, n = 0;
+    double best = 1e300;
+    for (int r = 2; r <= cap; n++) {
+        const int k = (ny + r - 1) / r; // strips of a column
+        const double t = cost((long)nsx * k, r);
+        if (t <= best) best = t, best_rows = r;
+        if (k == 1) break;
+        const int next = ((ny + k - 2) / (k - 1) + 1) & ~1; // the least even height with fewer
+        r = next > r ? next : r + 2;
+    }
+    if (tried) *tried = n + 1;
+    return best_rows;
+}
 cudaError_t launch_march(int mode, const ModelConst<float>& K, const StepLaunch& a,
                          cudaStream_t s);
 

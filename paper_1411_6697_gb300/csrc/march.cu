@@ -897,13 +897,11 @@ void march_plan(int mode, int nx, int ny, int* grid, int* strip_rows)
     const int nsx = (nx + BW - 1) / BW;
     const int even = (ny + 1) & ~1, cap = (mode & 8) && even > 64 ? 64 : even;
     int rows = 2;
-    double best = 1e300;
-    for (int r = 2; r <= cap && G > 0; r += 2) {
-        const long strips = (long)nsx * ((ny + r - 1) / r), rounds = (strips + G - 1) / G;
-        const double t = rounds * (r / 2 + MARCH_PROLOGUE) * (2 * strips <= G ? MARCH_ALONE : 1.0) +
-                         MARCH_TAIL * (r / 2);
-        if (t <= best) best = t, rows = r;
-    }
+    if (G > 0)
+        rows = march_rows(ny, cap, nsx, [&](long strips, int r) {
+            const long rounds = (strips + G - 1) / G;
+            return rounds * (r / 2 + MARCH_PROLOGUE) * (2 * strips <= G ? MARCH_ALONE : 1.0) + MARCH_TAIL * (r / 2);
+        });
     if (const char* env = getenv("LBKM_MARCH_ROWS")) { // tuning override (even)
         const int r = (atoi(env) + 1) & ~1;
         if (r >= 2) rows = r;
