@@ -568,8 +568,8 @@ __device__ __forceinline__ void recover32(const ModelConst<float>& K, const floa
         recover_one_f64_fast(m1.hi, m1.lo, r, pair_to_f64(m2.hi, m2.lo), pair_to_f64(m3.hi, m3.lo),
                              pair_to_f64(m4.hi, m4.lo), K.inv_DId, u, v, t);
         rho = m1.hi;
-        ux = d2f_fast(u);
-        uy = d2f_fast(v);
+        ux = m2.hi == 0.f ? 0.f : d2f_fast(u); // (f2d_fast(0) is 2^-127)
+        uy = m3.hi == 0.f ? 0.f : d2f_fast(v);
         T = d2f_fast(t);
         ig = dbits(t) > dbits(K.T_igd);
         ok = fabsf(m1.hi) <= FLT_MAX && fabsf(m2.hi) <= FLT_MAX && fabsf(m3.hi) <= FLT_MAX &&

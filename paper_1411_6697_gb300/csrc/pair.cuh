@@ -277,18 +277,20 @@ __device__ __forceinline__ float d2f_fast(double x)
 }
 __device__ __forceinline__ double df_to_f64_fast(float hi, float lo) { return f2d_fast(hi) + f2d_fast(lo); }
 
-// hi + lo rounded to binary64 on the integer pipe, for normalised pairs (|lo| at most a unit in
-// the last place of hi, the reciprocal seed's 2^-22 hi included): lo in units of the last place
-// of hi's binary64 image is added to that image as an integer. Below a power of two those units
-// halve. An FP64 addition would hold the FP64 unit for 64 cycles a warp.
+// hi + lo rounded to nearest in binary64 on the integer pipe, for normalised pairs (|lo| at most half
+// a unit in the last place of hi; hi zero or normal): lo in units of the last place of hi's binary64
+// image is added to that image as an integer. Those units are 2^-51 of lo 2^(128 - exponent of hi),
+// halved below a power of two; the power is one FP32 number over the whole range of hi, and the
+// product is small enough for any lo. An FP64 addition would hold the FP64 unit for 64 cycles a warp.
+// (The seed of a reciprocal, r + r e below, may lie a unit beside r: where it crosses a power of two
+// the sum is off by up to 2^-23, which the Newton step squares.)
 __device__ __forceinline__ double pair_to_f64(float hi, float lo)
 {
     const unsigned hb = __float_as_uint(hi);
-    const unsigned e = (306u << 23) - (hb & 0x7f800000u), top = 254u << 23; // 2^(52 - exponent of hi)
-    const float l = __uint_as_float(__float_as_uint(lo) ^ (hb & 0x80000000u));
-    int k = __float2int_rn(l * __uint_as_float(e < top ? e : top));
-    if ((hb & 0x7fffffu) == 0u && k < 0) k += k;
-    return __longlong_as_double(__double_as_longlong(f2d_fast(hi)) + k);
+    const float l = __uint_as_float(__float_as_uint(lo) ^ (hb & 0x80000000u)) *
+                    __uint_as_float(0x7f800000u - (hb & 0x7f800000u));
+    const float unit = (hb & 0x7fffffu) == 0u && l < 0.f ? 4503599627370496.f : 2251799813685248.f;
+    return __longlong_as_double(__double_as_longlong(f2d_fast(hi)) + __float2int_rn(l * unit));
 }
 
 // FP64 recovery of one cell with fewer FP64 operations: 1/m1 seeded by a double-float

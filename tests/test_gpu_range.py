@@ -31,3 +31,13 @@ def test_fp64_step_scales_with_the_density(nx, ny, tne, power):
     assert np.array_equal(g[:16], scale * f[:16])
     for a, b in zip(h, hs):
         assert np.array_equal(b, scale * a)
+
+
+@pytest.mark.parametrize("power", [-85, -60, 60, 90])
+@pytest.mark.parametrize("nx,ny", [(300, 1), (20000, 1), (70, 37), (700, 300)])
+def test_fp32_step_scales_with_the_density(nx, ny, power):
+    """Exact conserved sums at any density that leaves f and the sums' low parts (2^-24 of it) normal."""
+    scale = 2.0 ** power
+    f, _ = run(nx, ny, 0, 1.0, lbkm.F32)
+    g, _ = run(nx, ny, 0, scale, lbkm.F32)
+    assert np.array_equal(g[:16], np.float32(scale) * f[:16])
