@@ -504,24 +504,22 @@ __global__ void __launch_bounds__(ADJ_THREADS)
     }
 }
 
-// the objective's TNE term of one state alone: w_tne dx dt sum_x sum_k Delta_k^2
+// the objective's TNE term of one state alone: w_tne dx dt sum_x sum_k Delta_k^2, each Delta_k formed
+// as the reverse sweep forms it
 __global__ void __launch_bounds__(ADJ_THREADS)
-    adj_jtne(const ModelConst<double> K, const AdjArgs a)
+    adj_jtne(const __grid_constant__ ModelConst<double> K, const __grid_constant__ StepConst<double> E, const AdjArgs a)
 {
     __shared__ double sred[ADJ_THREADS / 32];
     const int nx = K.nx;
     double jt = 0.0;
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < nx; j += gridDim.x * blockDim.x) {
-        double f[16], m[16], q[16];
+        double f[16], m1, m2, m3, ux, uy, ux2, uy2, u2, T, D[TNE_K];
+        bool ok;
         for (int i = 0; i < 16; i++) f[i] = a.f[i * K.plane + j];
-        double rho, ux, uy, T; // as the macros kernel forms them for the reverse sweep
-        recover_f64(K.cd, K.wd, K.inv_DId, f, rho, ux, uy, T);
-        forward_moments(K, f, m);
-        feq_moments(K.DI, rho, ux, uy, T, q);
-        for (int k = 4; k < 16; k++) {
-            const double D = m[k] - q[k];
-            jt += D * D;
-        }
+        const Fly<double> b = butterflies(f);
+        recover64(K, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, ok);
+        deltas<true>(K, E, b, m1, m2, m3, ux, uy, ux2, uy2, u2, T, mu(m1, T), D);
+        for (int k = 0; k < TNE_K; k++) jt = fm(D[k], D[k], jt);
     }
     block_add(jt * a.jw, a.jacc, sred);
 }
@@ -617,7 +615,9 @@ cudaError_t launch_adj_seed(const ModelConst<double>& K, const AdjArgs& a, const
 
 cudaError_t launch_adj_jtne(const ModelConst<double>& K, const AdjArgs& a, int grid, cudaStream_t s)
 {
-    adj_jtne<<<grid, ADJ_THREADS, 0, s>>>(K, a);
+    StepConst<double> E;
+    step_const(K, &E);
+    adj_jtne<<<grid, ADJ_THREADS, 0, s>>>(K, E, a);
     return cudaGetLastError();
 }
 
