@@ -21,6 +21,7 @@ from __future__ import annotations
 import argparse
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -75,12 +76,22 @@ def measured_peak():
 
 
 # the FP32 2-D step runs march_kernel (march.cu); the FP64 2-D step tile_kernel (tile.cu)
-STEP_KERNEL_SOURCES = {
-    "march": ("march.cu", "pair.cuh", "vec2.cuh", "reduce.cuh", "cell.cuh", "kernels.cuh",
-              "model.h"),
-    "step": ("tile.cu", "cellops.cuh", "cell.cuh", "pair.cuh", "kernels.cuh", "model.h", "reduce.cuh"),
-    "batch": ("batch.cu", "cell.cuh", "pair.cuh", "vec2.cuh", "kernels.cuh", "model.h"),
-}
+STEP_KERNEL_FILE = {"march": "march.cu", "step": "tile.cu", "batch": "batch.cu"}
+
+
+def step_kernel_sources(kernel):
+    """The kernel's file and every file of the library that it includes, in alphabetical order."""
+    src = os.path.join(ROOT, "paper_1411_6697_gb300", "csrc")
+    found, todo = set(), [STEP_KERNEL_FILE[kernel]]
+    while todo:
+        f = todo.pop()
+        if f in found or not os.path.exists(os.path.join(src, f)):
+            continue
+        found.add(f)
+        todo += re.findall(r'^\s*#include "([^"]+)"', open(os.path.join(src, f)).read(), re.M)
+    return sorted(found)
+
+
 PROFILE = {"march": "march_kernel_reactive2d.md", "step": "step_kernel_fp64_reactive2d.md",
            "batch": "batch_kernel_batched.md"}
 
@@ -90,7 +101,7 @@ def step_kernel_digest(kernel="march"):
     import hashlib
     src = os.path.join(ROOT, "paper_1411_6697_gb300", "csrc")
     h = hashlib.sha256()
-    for f in STEP_KERNEL_SOURCES[kernel]:
+    for f in step_kernel_sources(kernel):
         h.update(open(os.path.join(src, f), "rb").read())
     return h.hexdigest()
 
