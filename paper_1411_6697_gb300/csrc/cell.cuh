@@ -17,33 +17,6 @@ __device__ __forceinline__ R rmin(R a, R b) { return a < b ? a : b; }
 template <typename R>
 __device__ __forceinline__ R rmax(R a, R b) { return a > b ? a : b; }
 
-// minmod of the NND scheme: 0 unless a and b share a sign, else the one of
-// smaller magnitude -- which is the median of a, b and 0, written as
-// max(min(a,b), min(max(a,b),0)).
-template <typename R>
-__device__ __forceinline__ R minmod(R a, R b)
-{
-    return rmax(rmin(a, b), rmin(rmax(a, b), R(0)));
-}
-
-// (H_{j+1/2} - H_{j-1/2}) / v of the NND flux of F = v q for v > 0, from
-// q_{j-2}, q_{j-1}, q_j, q_{j+1}: the interface value is q_j + mm(dq_j, dq_{j+1})/2.
-template <typename R>
-__device__ __forceinline__ R nnd_pos(R qm2, R qm1, R q0, R qp1)
-{
-    R d0 = qm1 - qm2, d1 = q0 - qm1, d2 = qp1 - q0;
-    return d1 + R(0.5) * (minmod(d1, d2) - minmod(d0, d1));
-}
-
-// the same for v < 0 from q_{j-1}, q_j, q_{j+1}, q_{j+2}: the interface value
-// is q_{j+1} - mm(dq_{j+1}, dq_{j+2})/2.
-template <typename R>
-__device__ __forceinline__ R nnd_neg(R qm1, R q0, R qp1, R qp2)
-{
-    R d1 = q0 - qm1, d2 = qp1 - q0, d3 = qp2 - qp1;
-    return d2 - R(0.5) * (minmod(d2, d3) - minmod(d1, d2));
-}
-
 // y = A x for an N x N block A of coefficients (type T) acting on lanes of type L
 // (a scalar, or a pair of cells packed for FFMA2).
 template <int N, typename T, typename L>
@@ -144,43 +117,6 @@ __device__ __forceinline__ void matvec_t(const T* A, const L* x, L* y)
 #pragma unroll
         for (int r = 1; r < N; r++) s = fma(A[r * N + c], x[r], s);
         y[c] = s;
-    }
-}
-
-// fb = M^T mb: the transpose of forward_moments, its steps reversed (moment placement,
-// sector blocks, the sector sums, the orbit butterflies), for the adjoint.
-template <typename R, typename L>
-__device__ __forceinline__ void forward_moments_t(const ModelConst<R>& K, const L* mb, L* fb)
-{
-    L pes[4] = {mb[0], mb[3], L(0.5) * (mb[4] + mb[6]), L(0.5) * (mb[13] + mb[15])};
-    L pea[2] = {L(0.5) * (mb[4] - mb[6]), L(0.5) * (mb[13] - mb[15])};
-    L px[4] = {mb[1], mb[7], mb[9], mb[11]}, py[4] = {mb[2], mb[8], mb[12], mb[10]};
-    L po[2] = {mb[5], mb[14]};
-    L es[4], ea[2], xo[4], yo[4], oo[2];
-    matvec_t<4>(K.Bes, pes, es);
-    matvec_t<2>(K.Bea, pea, ea);
-    matvec_t<4>(K.Bodd, px, xo);
-    matvec_t<4>(K.Bodd, py, yo);
-    matvec_t<2>(K.Boo, po, oo);
-    // axis orbits 0 (f0..f3) and 2 (f8..f11): es[a] = sx + sy, ea[a] = sx - sy
-#pragma unroll
-    for (int a = 0; a < 2; a++) {
-        const L sx = es[a] + ea[a], sy = es[a] - ea[a];
-        fb[8 * a + 0] = sx + xo[a];
-        fb[8 * a + 2] = sx - xo[a];
-        fb[8 * a + 1] = sy + yo[a];
-        fb[8 * a + 3] = sy - yo[a];
-    }
-    // diagonal orbits 1 (f4..f7) and 3 (f12..f15): e = s01 + s23, a_y = s01 - s23,
-    // a_x = d01 - d23, o = d01 + d23
-#pragma unroll
-    for (int d = 0; d < 2; d++) {
-        const L e = es[2 + d], ax = xo[2 + d], ay = yo[2 + d], o = oo[d];
-        const L s01 = e + ay, s23 = e - ay, d01 = ax + o, d23 = o - ax;
-        fb[4 + 8 * d + 0] = s01 + d01;
-        fb[4 + 8 * d + 1] = s01 - d01;
-        fb[4 + 8 * d + 2] = s23 + d23;
-        fb[4 + 8 * d + 3] = s23 - d23;
     }
 }
 
@@ -429,35 +365,6 @@ __device__ __forceinline__ int map_index(int j, int n, int bc)
 __host__ __device__ __forceinline__ int mirror_plane(int p)
 {
     return p == 16 ? 16 : (((p >> 2) & 1) ? ((p & ~3) | (3 - (p & 3))) : ((p & 1) ? (p ^ 2) : p));
-}
-
-// Value of plane p at (x, y) of the ghost-extended grid: inside the grid the stored
-// value; outside it the side's condition: periodic wrap, zero gradient (and walls,
-// corrected afterwards) copy the edge cell, Dirichlet gives the side's equilibrium,
-// specular mirrors the cell across the face with v_y reversed. A Dirichlet y side
-// wins in a corner (corner ghosts are never read by the cross-shaped stencils).
-template <typename R>
-__device__ __forceinline__ R ghost_value(const ModelConst<R>& K, const R* __restrict__ in, int p,
-                                         int x, int y)
-{
-    int sp = p;
-    if (y < 0 || y >= K.ny) {
-        const int s = y < 0 ? 2 : 3, code = K.sbc[s];
-        if (code == 3) return K.sfeq[s][p];
-        if (code == 4) {
-            y = y < 0 ? -y - 1 : 2 * K.ny - 1 - y;
-            y = y < 0 ? 0 : (y >= K.ny ? K.ny - 1 : y);
-            sp = mirror_plane(p);
-        } else {
-            y = map_index(y, K.ny, code == 0 ? 0 : 1);
-        }
-    }
-    if (x < 0 || x >= K.nx) {
-        const int s = x < 0 ? 0 : 1, code = K.sbc[s];
-        if (code == 3) return K.sfeq[s][p];
-        x = map_index(x, K.nx, code == 0 ? 0 : 1);
-    }
-    return in[sp * K.plane + (int64_t)y * K.pitch + x];
 }
 
 __device__ __forceinline__ float lane_recip(float x) { return 1.0f / x; }

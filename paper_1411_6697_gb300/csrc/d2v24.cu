@@ -1648,8 +1648,8 @@ cudaError_t launch_steps(const lbkm24* h, int from, int64_t& n, cudaStream_t st)
 
 // Steps per launch of split_kernel, or 0 where it does not apply: FP64, 1-D, moment form, no
 // records, and at most three windows an SM (a window's four warps use all of an SM's FP64 unit,
-// step_kernel's one warp a quarter). 5000 cells, two windows on some SMs: 37.1 us per step with
-// step_kernel, 21.6 with this.
+// step_kernel's one warp a quarter). us per step, this against step_kernel: 5000 and 8400 cells, two
+// windows on some or all SMs, 21.6 and 37; 9000 to 12700 cells, three, 24 to 28.1 and 37.
 int split_steps_for(const lbkm24* h, int sms)
 {
     if (h->p.precision != LBKM_F64 || h->p.ny != 1 || h->srt || h->p.tne_every > 0) return 0;

@@ -453,11 +453,11 @@ cudaError_t line_launch_t(const ModelConst<R>& K, const LinePlan& p, const LineA
 // an SM's FP64 units pass 3.0 us of warps one after another once its four quarters are busy
 // (us per step: w = 3 12.8, 4 13.9, 5 16.3, 6 17.5, 8 24.1, 16 44.7) and a launch costs
 // 1.5 us beside its steps. FP32: latency first, issue from about 20 warps on (w = 4 1.29,
-// 6 1.63, 8 1.93, 16 2.95, 230 40.5), a launch 2.0 us. So short grids take 16 steps per
-// launch (400 cells, FP32: 1.42 us per step against 3.3 with one), 16384 cells 4 steps of
-// 128 threads, one block per SM (FP32 1.80, FP64 14.2; 8 steps, whose 171 blocks no longer
-// fit one per SM, 2.19 and 23.3), and a million cells two FP32 steps (41.5; one 48.3, eight
-// 46.2), one FP64 step (622; four 683).
+// 6 1.63, 8 1.93, 16 2.95, 230 40.5), a launch 2.0 us. On 152 SMs that gives (threads x steps)
+// FP64 grids of a few thousand cells 96 x 16, 16384 cells 128 x 4 (14.2 us per step measured; 128 x 8,
+// whose 171 blocks no longer fit one per SM, 23.3), a million cells 192 x 1 (one step 622, four 683);
+// FP32 400 cells 64 x 8 (3.3 with one step), 16384 cells 160 x 8 (2.0 measured; 128 x 4 1.8 to 2.0), a
+// million cells 192 x 1.
 LinePlan line_plan(int precision, int nx, bool tne)
 {
     static int sms = -1;

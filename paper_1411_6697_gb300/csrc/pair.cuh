@@ -10,11 +10,6 @@
 
 namespace lbk {
 
-__device__ __forceinline__ void cp16(void* dst, const void* src)
-{
-    const unsigned s = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_wait()
@@ -196,58 +191,6 @@ __device__ __forceinline__ float d2f_rn(double x)
 // NaN), x > a exactly when the patterns compare so as signed 64-bit integers.
 __device__ __forceinline__ long long dbits(double x) { return __double_as_longlong(x); }
 
-// FP64 recovery: the exact conserved sums carried into FP64 (hi + lo), then rho,
-// u, T formed in FP64 arithmetic.
-// 1/m1 from an FP32 reciprocal refined by two FP64 Newton steps (each doubles the
-// correct bits: 22 -> 44 -> full FP64), then u and T in FP64.
-__device__ __forceinline__ void recover_one_f64(float seed_of, double m1, double m2, double m3,
-                                                double m4, double inv_DI, double& u, double& v,
-                                                double& t)
-{
-    double q = f2d_exact(rcp_approx(seed_of));
-    q = ::fma(q, ::fma(-m1, q, 1.0), q);
-    q = ::fma(q, ::fma(-m1, q, 1.0), q);
-    u = m2 * q;
-    v = m3 * q;
-    t = (m4 * q - (u * u + v * v)) * inv_DI;
-}
-
-__device__ __forceinline__ double df_to_f64(float hi, float lo) { return f2d_exact(hi) + f2d_exact(lo); }
-
-// rho, u, T of a cell pair from its 16 f: exact conserved sums, then FP64 (REC = 0)
-// or double-float (REC = 1); ig = T > T_ig decided in that precision, ok = rho > 0
-// and 0 < T < inf.
-template <int REC>
-__device__ __forceinline__ void recover_pair(const V2* f, const DfConst& C,
-                                             const ModelConst<float>& K, V2& rho, V2& ux, V2& uy,
-                                             V2& T, bool& ig0, bool& ig1, bool& ok0, bool& ok1)
-{
-    if constexpr (REC == 1) {
-        recover_pair_df(f, C, rho, ux, uy, T, ig0, ig1, ok0, ok1);
-    } else {
-        D2 m1, m2, m3, m4;
-        conserved_pair(f, C, m1, m2, m3, m4);
-        double u0, v0, t0, u1, v1, t1;
-        const double r0 = df_to_f64(m1.hi.x(), m1.lo.x());
-        const double r1 = df_to_f64(m1.hi.y(), m1.lo.y());
-        recover_one_f64(m1.hi.x(), r0, df_to_f64(m2.hi.x(), m2.lo.x()),
-                        df_to_f64(m3.hi.x(), m3.lo.x()), df_to_f64(m4.hi.x(), m4.lo.x()),
-                        K.inv_DId, u0, v0, t0);
-        recover_one_f64(m1.hi.y(), r1, df_to_f64(m2.hi.y(), m2.lo.y()),
-                        df_to_f64(m3.hi.y(), m3.lo.y()), df_to_f64(m4.hi.y(), m4.lo.y()),
-                        K.inv_DId, u1, v1, t1);
-        rho = m1.hi; // the exact sum rounded to FP32
-        ux = V2(d2f_rn(u0), d2f_rn(u1));
-        uy = V2(d2f_rn(v0), d2f_rn(v1));
-        T = V2(d2f_rn(t0), d2f_rn(t1));
-        const long long tig = dbits(K.T_igd), dmax = dbits(DBL_MAX);
-        ig0 = dbits(t0) > tig;
-        ig1 = dbits(t1) > tig;
-        ok0 = dbits(r0) > 0 && dbits(t0) > 0 && dbits(t0) <= dmax;
-        ok1 = dbits(r1) > 0 && dbits(t1) > 0 && dbits(t1) <= dmax;
-    }
-}
-
 // Branch-free forms of the two conversions, for the values a step's recovery produces
 // (normal binary32 / binary64 numbers of modest size, or zero):
 // f2d_fast moves the IEEE-754 fields of a normal binary32 value into binary64 exactly
@@ -310,7 +253,8 @@ __device__ __forceinline__ void recover_one_f64_fast(float m1h, float m1l, doubl
     t = ::fma(-m3, v, ::fma(-m2, u, m4)) * (q * inv_DI);
 }
 
-// recover_pair with the branch-free conversions; cells whose conserved sums are not
+// rho, u, T of a cell pair from its 16 f: exact conserved sums, then FP64 (REC = 0) or
+// double-float (REC = 1); ig = T > T_ig decided in that precision. Cells whose conserved sums are not
 // finite in FP32 are flagged before anything is converted.
 template <int REC>
 __device__ __forceinline__ void recover_pair_fast(const V2* f, const DfConst& C,

@@ -34,13 +34,6 @@ __device__ __forceinline__ R warp_max(R v)
     return v;
 }
 
-template <typename R>
-__device__ __forceinline__ R big_value();
-template <>
-__device__ __forceinline__ float big_value<float>() { return FLT_MAX; }
-template <>
-__device__ __forceinline__ double big_value<double>() { return DBL_MAX; }
-
 // Last block of a launch: reduce the per-block partials (fixed order) into a
 // TNE record. Called by every thread of that block.
 // Partials are stored quantity-major: partial q of block b at partials[q * nblocks + b].
