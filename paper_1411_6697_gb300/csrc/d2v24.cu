@@ -15,7 +15,7 @@
 // 720 of its instructions per warp and 1-D step, 240 more where a cell of the warp reacts.
 // Measured per step, against one thread per cell reading its stencil through the cache, every
 // sum normalised, the reaction in FP64 divisions and exponentials throughout: 2048^2 FP32 1.95
-// -> 0.60 ms, the 5000-cell detonation FP64 54 -> 37 us, FP32 12.6 -> 6.6 us.
+// -> 0.67 ms, the 5000-cell detonation FP64 54 -> 37 us, FP32 12.6 -> 6.6 us.
 //
 // M and M^-1 act in block form: butterflies inside each orbit of four velocities
 // (axis: f1+f3, f2+f4, f1-f3, f2-f4; diagonal: the sum and the three sign patterns)
