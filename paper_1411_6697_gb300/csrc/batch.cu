@@ -17,7 +17,7 @@
 // thread 0.430; one cell and two steps 0.330 (four 0.361: the shared edges grow; five or eight
 // blocks an SM 0.356, 0.333); with the pairs joined on the integer pipe (pair_to_f64) 0.315 (one
 // step 0.367, three 0.329), with the even moments' equilibria rounded before they are subtracted
-// (deltas, cellops.cuh) 0.322.
+// (deltas, cellops.cuh) 0.322, and with pair_to_f64's one select before the rounding 0.314.
 #include <float.h>
 #include <stdint.h>
 
